@@ -58,9 +58,9 @@ def listed():
         # the Holstein benchmark: one orbital, a phonon mode cut off at ten quanta
         {"name": "phonon_norb1_ns12_nph10_fp32", "kind": "phonon", "norb": 1, "nbath": 11,
          "nup": 6, "ndw": 6, "precision": "fp32", "nph": 10},
-        # a ground state with its vector at the two-orbital benchmark size
-        {"name": "ground_norb2_ns16_fp32", "kind": "ground", "norb": 2, "nbath": 7, "nup": 8,
-         "ndw": 8, "precision": "fp32"},
+        # a two-orbital ground state with its vector in the default precision
+        {"name": "ground_norb2_ns14_fp64", "kind": "ground", "norb": 2, "nbath": 6, "nup": 7,
+         "ndw": 7, "precision": "fp64"},
         # the Green's function of one orbital in the default precision
         {"name": "chain_norb2_ns12_fp64", "kind": "chain", "norb": 2, "nbath": 5, "nup": 6,
          "ndw": 5, "precision": "fp64"},
@@ -95,9 +95,9 @@ def draw(rng):
              "nup": ns // 2 + rng.randint(-2, 1), "ndw": ns // 2 + rng.randint(-2, 1),
              "precision": rng.choice(["fp32", "fp64"]), "nph": rng.randint(1, 10)}
     elif kind == "ground":
-        ns, norb = shape(8, 15, (1, 2, 3))
+        ns, norb = shape(8, 14, (1, 2, 3))
         c = {"kind": "ground", "norb": norb, "nbath": ns // norb - 1, "nup": (ns + 1) // 2,
-             "ndw": ns // 2, "precision": "fp32" if ns > 12 else rng.choice(["fp32", "fp64"])}
+             "ndw": ns // 2, "precision": "fp64"}
     elif kind == "chain":
         ns, norb = shape(8, 12, (1, 2, 3))
         c = {"kind": "chain", "norb": norb, "nbath": ns // norb - 1,
@@ -106,6 +106,7 @@ def draw(rng):
         ns, norb = shape(8, 10, (1, 2, 3))
         c = {"kind": "solve", "norb": norb, "nbath": ns // norb - 1,
              "nup": ns // 2 + rng.randint(-1, 1), "ndw": ns // 2, "precision": "fp64"}
+    c["U"] = round(rng.uniform(1.0, 5.0), 3)
     return {k: v for k, v in c.items() if k != "name"}
 
 
@@ -114,7 +115,8 @@ def draw(rng):
 def _model(case, seed):
     norb, nbath = case["norb"], case["nbath"]
     r = np.random.RandomState((seed * 7919 + 17) % (1 << 31))
-    U, J = (2.0, 0.0) if norb == 1 else (2.5, 0.4)
+    U = case.get("U", 2.0 if norb == 1 else 2.5)
+    J = 0.0 if norb == 1 else 0.16 * U
     Ust = U - 2.0 * J
     e_d = -0.5 * (U + (norb - 1) * (2.0 * Ust - J))
     one = np.ones((2, 1, 1))
@@ -189,7 +191,7 @@ def run(st):
 # ------------------------------------------------------------------ work
 
 #: Steps a ground state takes at these sizes (each reads one vector and writes one).
-GROUND_STEPS = {"fp32": 60, "fp64": 90}
+GROUND_STEPS = 90
 
 
 def work(case):
@@ -211,11 +213,11 @@ def work(case):
         n = dim * (case["nph"] + 1)
         return {"bytes": 2 * size * n, "flops": (flops + 7.0) * n}
     if kind == "ground":
-        k = GROUND_STEPS[case["precision"]]
+        k = GROUND_STEPS
         return {"bytes": k * 2 * size * dim, "flops": k * (flops + 8.0) * dim}
     # chains: every step one product and the recurrence on a sector next to this one
     chains = 2 if kind == "chain" else 2 * case["norb"] * (1 if case["nup"] == case["ndw"] else 2)
-    steps = GF_STEPS * chains + (0 if kind == "chain" else GROUND_STEPS[case["precision"]])
+    steps = GF_STEPS * chains + (0 if kind == "chain" else GROUND_STEPS)
     return {"bytes": steps * 2 * size * dim, "flops": steps * (flops + 8.0) * dim}
 
 
