@@ -28,6 +28,7 @@ import torch
 import paper_2105_06806_gb300 as ed
 
 BETA, NMATS, GF_STEPS = 100.0, 512, 200
+TOL = 1e-10  # Ritz residual of the ground states
 DTYPE = {"fp64": torch.float64, "fp32": torch.float32}
 
 
@@ -106,7 +107,7 @@ def draw(rng):
         ns, norb = shape(8, 10, (1, 2, 3))
         c = {"kind": "solve", "norb": norb, "nbath": ns // norb - 1,
              "nup": ns // 2 + rng.randint(-1, 1), "ndw": ns // 2, "precision": "fp64"}
-    c["U"] = round(rng.uniform(1.0, 5.0), 3)
+    c["U"] = round(rng.uniform(1.0, 3.0), 3)
     return {k: v for k, v in c.items() if k != "name"}
 
 
@@ -163,7 +164,7 @@ def prepare(case, seed):
         st["psi"] = torch.zeros(s.dim, dtype=DTYPE[p], device="cuda")
     elif kind == "chain":
         st["psi"] = torch.zeros(s.dim, dtype=DTYPE[p], device="cuda")
-        st["e0"] = ed.lanczos_ground(s, p, psi=st["psi"])["e0"]
+        st["e0"] = ed.lanczos_ground(s, p, psi=st["psi"], tol=TOL)["e0"]
     return st
 
 
@@ -178,13 +179,13 @@ def run(st):
         ed.eph_matvec(st["sector"], st["ph"], st["v"], st["w"], p)
         return st["w"]
     if kind == "ground":
-        r = ed.lanczos_ground(st["sector"], p, psi=st["psi"])
+        r = ed.lanczos_ground(st["sector"], p, psi=st["psi"], tol=TOL)
         return {"e0": r["e0"], "psi": st["psi"]}
     if kind == "chain":
         G, info = ed.gf_lanczos(st["sector"], st["psi"], st["e0"], 0, 0, p, GF_STEPS, BETA, NMATS)
         return {"G": G, "weights": [info["weight_particle"], info["weight_hole"]]}
     r, G = ed.solve(st["model"], case["nup"], case["ndw"], precision=p, nmats=NMATS, beta=BETA,
-                    gf_steps=GF_STEPS)
+                    gf_steps=GF_STEPS, tol=TOL)
     return {"e0": r["e0"], "G": G}
 
 
