@@ -1,0 +1,10 @@
+// Instances of the orbital-factorised product (fiber.cuh), split over
+// translation units so that they compile in parallel.
+#include "fiber.cuh"
+
+namespace fiber {
+template ed_status launch_g<2>(const HvLaunch<float> *, int, cudaStream_t);
+template ed_status launch_g<3>(const HvLaunch<float> *, int, cudaStream_t);
+template ed_status launch_g<4>(const HvLaunch<float> *, int, cudaStream_t);
+template ed_status launch_g<5>(const HvLaunch<float> *, int, cudaStream_t);
+}  // namespace fiber

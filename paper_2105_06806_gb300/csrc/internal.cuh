@@ -121,7 +121,9 @@ struct BlockInfo {
 struct HvItem {
   int32_t r0, nr, c0, nc;  // rows [r0, r0+nr) x columns [c0, c0+nc), one block pair
   int32_t c0p;             // first column in the vector layout (padded in block-major)
-  int32_t deg;             // ELL width of the up block (block-major), 0: use CSR
+  int32_t deg;             // ELL width of the up block (block-major), 0: use CSR;
+                           // orbital-factorised product: its group occupations, 4 bits
+                           // each, and the CTA shape from bit 24
   int32_t ell_off;         // first ELL entry of the up block
   int32_t ncp;             // ELL row length (padded block width)
 };
@@ -137,6 +139,8 @@ struct ItemList {
   HvItem *d_items = nullptr;
   int64_t nitems = 0;
   size_t smem = 0;
+  int fiber = 0;               // group size of the orbital-factorised product, 0: not used
+  int64_t fiber_n[2] = {0, 0};  // its items per CTA shape (the list is in that order)
   DwItem *d_ditems = nullptr;  // non-null: two-pass product (block pairs larger than L2)
   int64_t nditems = 0;
 };
@@ -317,6 +321,11 @@ struct HvTables {
   int64_t small_grid;      // its CTAs (= block partials of the Lanczos mode)
   int32_t small_chunk;     // its elements per thread
   bool passa_wide;         // two-pass product: the wide shape of the H_up pass
+  // orbital-factorised product (fiber.cuh): group size, 0 where not used; items
+  // per CTA shape; hop amplitudes of orbital k at hop_up[k (G - 1) + level]
+  int fiber = 0;
+  int64_t fiber_n[2] = {0, 0};
+  T hop_up[ED_MAX_NS];
   // H_nd (spin exchange, pair hopping): move tables of this layout, or null
   const int32_t *nd_up = nullptr, *nd_dw = nullptr;
   int64_t nd_ncols = 0;
@@ -376,6 +385,17 @@ template <typename T>
 ed_status ed_launch_nd(const HvTables<T> &tb, int mode, const T *v, T *w, T *const *bufs,
                        T *const *basis, const struct LanczosState *state, double *part,
                        cudaStream_t st);
+// Orbital-factorised FP32 product (fiber.cuh): groups of FIBER_MIN_G ..
+// FIBER_MAX_G levels; items of at most FIBER_ROWS rows in one of two CTA
+// shapes, each with room for FIBER_CAP elements of v.
+constexpr int FIBER_MIN_G = 2, FIBER_MAX_G = 8, FIBER_ROWS = 64, FIBER_MAX_W_NORB = 5;
+constexpr int FIBER_SHAPES = 2;
+constexpr int FIBER_CAP[FIBER_SHAPES] = {4912, 9024};
+// shapes compiled for a group size (bit s): blocks too wide for them do not
+// occur in a sector whose vectors fit the device
+constexpr int fiber_shapes(int g) {
+  return g >= 4 && g <= 6 ? 1 | 1 << 1 : 1;
+}
 // layout 0: sector (paper) order; 1: block-major order
 template <typename T>
 HvTables<T> ed_hv_tables(ed_sector s, int layout);

@@ -961,7 +961,7 @@ static ed_status second_pass(ed_sector s, const HvTables<T> &tb, T *const *bufs,
   // then the streaming update, which here also adds y_j v_j into psi) instead
   // of the fused second-pass H_dw epilogue: 14.3 + 3 ms against 19.6 ms per
   // step at Ns=18; the same operations, so the same vectors bit for bit.
-  const bool split = tb.ditems && !tb.small_cols;
+  const bool split = (tb.ditems || tb.fiber) && !tb.small_cols;
   for (int j = j0; j + 1 < k; ++j) {
     if (split) {
       int64_t np1 = 0;

@@ -24,30 +24,7 @@
 #include <mutex>
 #include <type_traits>
 
-#include "internal.cuh"
-
-template <typename T>
-__device__ __forceinline__ T fma_t(T a, T b, T c);
-template <>
-__device__ __forceinline__ float fma_t<float>(float a, float b, float c) {
-  return __fmaf_rn(a, b, c);
-}
-template <>
-__device__ __forceinline__ double fma_t<double>(double a, double b, double c) {
-  return __fma_rn(a, b, c);
-}
-template <typename T>
-__device__ __forceinline__ T mul_t(T a, T b);
-template <>
-__device__ __forceinline__ float mul_t<float>(float a, float b) { return __fmul_rn(a, b); }
-template <>
-__device__ __forceinline__ double mul_t<double>(double a, double b) { return __dmul_rn(a, b); }
-template <typename T>
-__device__ __forceinline__ T add_t(T a, T b);
-template <>
-__device__ __forceinline__ float add_t<float>(float a, float b) { return __fadd_rn(a, b); }
-template <>
-__device__ __forceinline__ double add_t<double>(double a, double b) { return __dadd_rn(a, b); }
+#include "product.cuh"
 
 // Register tile: 4 consecutive columns x RT rows; the RT rows of one column
 // form one 16-byte vector in shared memory (FP32: RT = 4, or 2 with an
@@ -99,30 +76,6 @@ constexpr int rt_passa() { return sizeof(T) == 4 && WIDE ? 4 : 2; }
 template <bool WIDE>
 constexpr int passa_threads() { return WIDE ? 1024 : 512; }
 
-// four consecutive values of a 16-byte aligned row segment
-__device__ __forceinline__ void load4(const float *p, float *y) {
-  const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-  y[0] = v.x;
-  y[1] = v.y;
-  y[2] = v.z;
-  y[3] = v.w;
-}
-__device__ __forceinline__ void load4(const double *p, double *y) {
-  const double2 a = __ldg(reinterpret_cast<const double2 *>(p));
-  const double2 b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-  y[0] = a.x;
-  y[1] = a.y;
-  y[2] = b.x;
-  y[3] = b.y;
-}
-
-__device__ __forceinline__ void store4(float *p, const float *y) {
-  *reinterpret_cast<float4 *>(p) = make_float4(y[0], y[1], y[2], y[3]);
-}
-__device__ __forceinline__ void store4(double *p, const double *y) {
-  reinterpret_cast<double2 *>(p)[0] = make_double2(y[0], y[1]);
-  reinterpret_cast<double2 *>(p)[1] = make_double2(y[2], y[3]);
-}
 __device__ __forceinline__ void vec_get(const float4 &v, float *x) {
   x[0] = v.x;
   x[1] = v.y;
@@ -175,6 +128,24 @@ static int64_t small_grid_of(int64_t n) {
 }
 
 static bool passa_is_wide(ed_sector s);
+
+// fiber.cuh: launch of the orbital-factorised product (a = nullptr: prepare)
+namespace fiber {
+template <int G>
+ed_status launch_g(const HvLaunch<float> *a, int mode, cudaStream_t st);
+}
+static ed_status launch_fiber(int g, const HvLaunch<float> *a, int mode, cudaStream_t st) {
+  switch (g) {
+    case 2: return fiber::launch_g<2>(a, mode, st);
+    case 3: return fiber::launch_g<3>(a, mode, st);
+    case 4: return fiber::launch_g<4>(a, mode, st);
+    case 5: return fiber::launch_g<5>(a, mode, st);
+    case 6: return fiber::launch_g<6>(a, mode, st);
+    case 7: return fiber::launch_g<7>(a, mode, st);
+    case 8: return fiber::launch_g<8>(a, mode, st);
+  }
+  return ED_ERR_ARG;
+}
 
 template <typename T>
 static void fill_tables(HvTables<T> &t, const SpinTables &u, const SpinTables &d, const T *vu,
@@ -247,21 +218,12 @@ HvTables<float> ed_hv_tables<float>(ed_sector s, int layout) {
   t.small_grid = t.small_cols ? small_grid_of(s->bdim) : 0;
   t.small_chunk = (int32_t)small_chunk_of(s->bdim);
   t.passa_wide = layout == 1 && passa_is_wide(s);
+  t.fiber = il.fiber;
+  for (int k = 0; k < FIBER_SHAPES; ++k) t.fiber_n[k] = il.fiber_n[k];
+  for (int l = 0; l + s->mp.norb < s->mp.ns; ++l) t.hop_up[l] = (float)s->mp.V[0][s->mp.norb + l];
   set_nd<float>(t, s, layout);
   return t;
 }
-
-template <typename T>
-struct HvLaunch {
-  HvTables<T> tb;
-  const T *v;
-  T *w;
-  T *b0, *b1, *b2;
-  T *const *basis;  // Lanczos mode: vector j at basis[j] (else b[j % 3])
-  T *psi;
-  LanczosState *st;
-  double *part;
-};
 
 constexpr int HV_THREADS = 512;
 // H_dw pass of the two-pass product (k_hv_dw)
@@ -471,8 +433,31 @@ static bool passa_is_wide(ed_sector s) {
   return w > (int64_t)EDGB_PASSA_WIDE;
 }
 
+// CTA shape of the orbital-factorised product for an up block of padded width
+// w: the smallest one with room for a row; -1: none
+static int fiber_shape(int g, int64_t w) {
+  for (int k = 0; k < FIBER_SHAPES; ++k)
+    if (((fiber_shapes(g) >> k) & 1) && w <= FIBER_CAP[k]) return k;
+  return -1;
+}
+
+// Products (ms) of the orbital-factorised pass with the H_dw pass against the
+// kernels it replaces in the tiled family: Norb=3 Ns=18 14.7 / 24.9, Norb=2
+// Ns=16 0.96 / 1.13, Norb=3 Ns=15 0.31 / 0.45, Norb=4 Ns=16 1.28 / 1.84; the
+// autotuner still compares the family with the element-parallel kernel.
+// Group size of the orbital-factorised product where the sector's FP32
+// block-major product can take it, else 0: one orbital has no factorisation,
+// and a row of every up block has to fit a CTA.
+static int fiber_group(ed_sector s) {
+  const int g = s->mp.nbath + 1;
+  if (s->mp.norb < 2 || g < FIBER_MIN_G || g > FIBER_MAX_G) return 0;
+  for (size_t k = 0; k + 1 < s->up_off_pad.size(); ++k)
+    if (fiber_shape(g, s->up_off_pad[k + 1] - s->up_off_pad[k]) < 0) return 0;
+  return g;
+}
+
 static ed_status build_dw_items(ed_sector s, ItemList &il, int elem, cudaStream_t cs) {
-  if (il.d_ditems || !two_pass_wanted(s, elem)) return ED_OK;
+  if (il.d_ditems || (!il.fiber && !two_pass_wanted(s, elem))) return ED_OK;
   const std::vector<int64_t> &ob_dw = s->bi[1].offset, &ob_up = s->bi[0].offset;
   std::vector<DwItem> items;
   for (size_t bd = 0; bd + 1 < ob_dw.size(); ++bd) {
@@ -670,6 +655,7 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
                                     : (wide ? rt_passa<double, true>() : rt_passa<double, false>()))
                        : (elem == 4 ? Tile<float>::RT : Tile<double>::RT);
   const int threads = passa ? (wide ? passa_threads<true>() : passa_threads<false>()) : HV_THREADS;
+  const int fiber = layout == 1 && elem == 4 ? fiber_group(s) : 0;
   std::vector<HvItem> items;
   size_t smem = 0;
   for (size_t bd = 0; bd + 1 < ob_dw.size(); ++bd) {
@@ -688,13 +674,26 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
       R = std::min<int64_t>(std::min<int64_t>(R, HV_MAXROWS), R1 - R0);
       const size_t need = (size_t)((R + RT - 1) / RT) * per_group;
       if (need <= HV_SMEM_MAX) smem = std::max(smem, need);
-      const int32_t deg = layout == 0 ? 0 : s->ell_deg[bu];
+      int32_t deg = layout == 0 ? 0 : s->ell_deg[bu];
+      if (fiber) {
+        const int64_t pitch = round_up(nc, 4);
+        const int shape = fiber_shape(fiber, pitch);
+        R = std::min<int64_t>(std::min<int64_t>(FIBER_CAP[shape] / pitch, FIBER_ROWS), R1 - R0);
+        deg = shape << 24;
+        for (int k = 0; k < s->mp.norb; ++k)
+          deg |= (int32_t)s->bi[0].keys[bu * s->mp.norb + k] << (4 * k);
+      }
       const int32_t eoff = layout == 0 ? 0 : s->ell_off[bu];
       const int32_t ncp = (int32_t)(op_up[bu + 1] - op_up[bu]);
       for (int64_t r = R0; r < R1; r += R)
         items.push_back(HvItem{(int32_t)r, (int32_t)std::min<int64_t>(R, R1 - r), (int32_t)C0,
                                (int32_t)nc, (int32_t)op_up[bu], deg, eoff, ncp});
     }
+  }
+  if (fiber) {
+    std::stable_sort(items.begin(), items.end(),
+                     [](const HvItem &x, const HvItem &y) { return x.deg >> 24 < y.deg >> 24; });
+    for (const HvItem &x : items) ++il.fiber_n[x.deg >> 24];
   }
   HvItem *d_items = nullptr;
   ED_TRY(ed_dmalloc((void **)&d_items, std::max<size_t>(items.size(), 1) * sizeof(HvItem), cs,
@@ -712,6 +711,7 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
   // published only once complete
   il.nitems = (int64_t)items.size();
   il.smem = smem;
+  il.fiber = fiber;
   il.d_items = d_items;
   s->device_bytes += (int64_t)(items.size() * sizeof(HvItem));
   if (layout == 1) {
@@ -719,19 +719,6 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
     ED_TRY(decide_kernel(s, elem, cs));
   }
   return ED_OK;
-}
-
-template <typename T>
-__device__ __forceinline__ double block_sum(double x, double *red) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = x;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += red[k];
-  }
-  return s;
 }
 
 // Slot of column c in a staged row group of ncp = 4 q4 columns: columns are
@@ -744,21 +731,6 @@ __device__ __forceinline__ int stage_pos(int c, int q4) { return (c & 3) * q4 + 
 // One tile: 4 consecutive columns cb..cb+3 x RT rows of the thread's row
 // group.  FULL: all RT rows exist and all 4 columns are inside the block
 // (no predication).  BLK: block-major layout (ELL table, aligned vectors).
-// Asynchronous copy of one element from global to shared memory (cp.async,
-// cached in L1), so that all the loads of a staging loop are in flight at
-// once instead of each waiting in a register for its shared-memory store.
-template <typename T>
-__device__ __forceinline__ void cp_async_elem(T *dst_smem, const T *src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst_smem);
-  if (sizeof(T) == 8)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
-}
-
 template <typename T, bool FULL, bool BLK, bool NODW, int RTX>
 __device__ __forceinline__ void hv_tile(const HvTables<T> &tb, const HvItem &it, const T *g,
                                         const T *smq, bool staged, int lr0, int nrt, int cb,
@@ -1389,6 +1361,8 @@ ed_status ed_hv_prepare() {
   if (dev < 64 && done[dev]) return ED_OK;
   ED_TRY((prepare_layout<T, false>()));
   ED_TRY((prepare_layout<T, true>()));
+  if (sizeof(T) == 4)
+    for (int g = FIBER_MIN_G; g <= FIBER_MAX_G; ++g) ED_TRY(launch_fiber(g, nullptr, 0, nullptr));
   if (dev < 64) done[dev] = true;
   return ED_OK;
 }
@@ -1402,6 +1376,11 @@ static ed_status launch_mode(const HvLaunch<T> &a, cudaStream_t st) {
       k_hv_small<T, MODE, true><<<(unsigned)a.tb.small_grid, HVS_THREADS, 0, st>>>(a);
     else
       k_hv_small<T, MODE, false><<<(unsigned)a.tb.small_grid, HVS_THREADS, 0, st>>>(a);
+  } else if (a.tb.fiber) {
+    if constexpr (sizeof(T) == 4) {
+      ED_TRY(launch_fiber(a.tb.fiber, &a, MODE, st));
+    }
+    k_hv_dw<T, MODE><<<(unsigned)a.tb.nditems, DW_THREADS, 0, st>>>(a);
   } else if (a.tb.ditems) {
     if (a.tb.passa_wide)
       k_hv<T, MODE, true, true, rt_passa<T, true>(), passa_threads<true>()>
@@ -1427,7 +1406,10 @@ ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v,
   ED_TRY(ed_hv_prepare<T>());
   HvLaunch<T> a;
   a.tb = tb;
-  if (nparts) *nparts = tb.small_cols ? tb.small_grid : (tb.ditems ? tb.nditems : tb.nitems);
+  // CTAs of the (last) product kernel = its partial sums in the Lanczos mode
+  const int64_t np = tb.small_cols ? tb.small_grid
+                                   : (tb.ditems ? tb.nditems : tb.nitems);
+  if (nparts) *nparts = np;
   if (tb.nitems == 0 || tb.dup == 0) return ED_OK;
   if (!tb.items) return ED_ERR_ARG;
   a.v = v;
@@ -1444,7 +1426,6 @@ ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v,
   else ED_TRY((launch_mode<T, HV_SECOND>(a, st)));
   if (!tb.nd_up) return ED_OK;
   // spin exchange and pair hopping, added to the product (partials after the product's)
-  const int64_t np = tb.small_cols ? tb.small_grid : (tb.ditems ? tb.nditems : tb.nitems);
   if (nparts) *nparts = np + ed_nd_grid(tb.ddw, tb.nd_ncols);
   return ed_launch_nd<T>(tb, mode, v, w, bufs, basis, state, part ? part + np : nullptr, st);
 }
@@ -1503,7 +1484,7 @@ static ed_status kernel_of(ed_sector s, ed_precision prec, int *e, int32_t *kern
   ED_TRY(ed_build_items(s, 1, elem));
   *kernel = s->hv_kernel[*e] == 1
                 ? ED_KERNEL_ELEMENTWISE
-                : (s->items[1][*e].d_ditems ? ED_KERNEL_TWO_PASS : ED_KERNEL_TILED);
+                : (two_pass_wanted(s, elem) ? ED_KERNEL_TWO_PASS : ED_KERNEL_TILED);
   return ED_OK;
 }
 
@@ -1536,7 +1517,7 @@ extern "C" ed_status ed_sector_set_kernel(ed_sector s, ed_precision prec, int32_
     s->hv_kernel[e] = 1;
   } else if (kernel == ED_KERNEL_TILED || kernel == ED_KERNEL_TWO_PASS) {
     // the tiled family: one or two passes as the sector's size decides
-    if ((kernel == ED_KERNEL_TWO_PASS) != (s->items[1][e].d_ditems != nullptr)) {
+    if ((kernel == ED_KERNEL_TWO_PASS) != two_pass_wanted(s, e ? 8 : 4)) {
       ed_set_error_msg("one or two passes is fixed by the sector's block sizes");
       return ED_ERR_UNSUPPORTED;
     }

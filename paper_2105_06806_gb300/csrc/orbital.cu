@@ -131,6 +131,10 @@ ed_status view_tables(ed_sector s, const OrbView &v, Mem &store, HvTables<T> *tb
   *tb = ed_hv_tables<T>(s, 1);
   tb->items = d_items;
   tb->nitems = (int64_t)keep.size();
+  if (tb->fiber) {
+    for (int64_t &n : tb->fiber_n) n = 0;
+    for (const HvItem &it : keep) ++tb->fiber_n[it.deg >> 24];
+  }
   tb->ditems = il.d_ditems ? d_ditems : nullptr;
   tb->nditems = il.d_ditems ? (int64_t)dkeep.size() : 0;
   tb->small_cols = nullptr;  // the tiled family: the items carry the block pair
