@@ -279,6 +279,11 @@ __device__ __forceinline__ int fast_div(int i, float inv) {
   return __float2int_rz(((float)i + 0.5f) * inv);
 }
 
+// Item: rows r0 .. r0 + nr of one up block.
+struct FibItem {
+  int r0, nr, c0, nc, c0p, deg;
+};
+
 struct RowData {
   const float *ed;     // [rows] E_dw
   const uint8_t *md;   // [rows] impurity mask
@@ -286,7 +291,7 @@ struct RowData {
 };
 
 template <int G, int N, int KIND, typename T>
-__device__ __forceinline__ void step_n(const HvTables<T> &tb, const HvItem &it, T *X, T *A, int k,
+__device__ __forceinline__ void step_n(const HvTables<T> &tb, const FibItem &it, T *X, T *A, int k,
                                        int S, int parity, const RowData &rd) {
   constexpr int L = binom(G, N);
   if constexpr (KIND >= STEP_EMPTY && (N == 0 || N == G)) return;
@@ -320,7 +325,7 @@ __device__ __forceinline__ void step_n(const HvTables<T> &tb, const HvItem &it, 
 }
 
 template <int G, int KIND, typename T, int N = 0>
-__device__ __forceinline__ void step(int n, const HvTables<T> &tb, const HvItem &it, T *X, T *A,
+__device__ __forceinline__ void step(int n, const HvTables<T> &tb, const FibItem &it, T *X, T *A,
                                      int k, int S, int parity, const RowData &rd) {
   if (n == N) {
     step_n<G, N, KIND, T>(tb, it, X, A, k, S, parity, rd);
@@ -329,17 +334,18 @@ __device__ __forceinline__ void step(int n, const HvTables<T> &tb, const HvItem 
   }
 }
 
-// H_up pass: one item (rows of one dw block x one up block) per CTA; the
+// H_up pass: one item (rows x one up block) per CTA; the
 // diagonal and H_up, written unscaled (k_hv_dw adds H_dw).  lanczos: the
 // vectors of the recurrence (step j of the device state) instead of a.v, a.w.
 template <int G, int SHAPE>
 __global__ void __launch_bounds__(Shape<G, SHAPE>::NT, Shape<G, SHAPE>::CTAS)
-    k_hv_fiber(HvLaunch<float> a, int64_t first, int lanczos) {
+    k_hv_fiber(HvLaunch<float> a, int lanczos) {
   constexpr int CAP = Shape<G, SHAPE>::CAP, NT = Shape<G, SHAPE>::NT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float *const X = reinterpret_cast<float *>(smem_raw), *const A = X + CAP;
   __shared__ float s_ed[FIBER_ROWS], s_w[1 << (2 * FIBER_MAX_W_NORB)];
   __shared__ uint8_t s_md[FIBER_ROWS];
+  __shared__ FibItem s_it;
   const HvTables<float> &tb = a.tb;
   const float *g = a.v;
   float *out = a.w;
@@ -354,7 +360,31 @@ __global__ void __launch_bounds__(Shape<G, SHAPE>::NT, Shape<G, SHAPE>::CTAS)
       out = a.basis[j + 1];
     }
   }
-  const HvItem it = tb.items[first + blockIdx.x];
+  // the item's up block: the last one whose first item is not above this item
+  if (threadIdx.x < 32) {
+    FibItem it;
+    const int item = (int)(tb.fib_first[SHAPE] + blockIdx.x);
+    const FibBlock *fb = tb.fib[SHAPE];
+    int b = 0;
+    for (int q = 0; q < tb.nfib[SHAPE]; q += 32) {
+      const int lane = q + (int)(threadIdx.x & 31);
+      const unsigned le =
+          __ballot_sync(0xffffffffu, lane < tb.nfib[SHAPE] && fb[lane].first <= item);
+      if (!le) break;
+      b = q + 31 - __clz(le);
+    }
+    const FibBlock blk = fb[b];
+    it.c0 = blk.c0;
+    it.nc = blk.nc;
+    it.c0p = blk.c0p;
+    it.deg = blk.keys;
+    const int64_t r = (int64_t)(item - blk.first) * blk.rows;
+    it.r0 = (int)(tb.row0 + r);
+    it.nr = (int)min((int64_t)blk.rows, tb.rows - r);
+    if (threadIdx.x == 0) s_it = it;
+  }
+  __syncthreads();
+  const FibItem &it = s_it;
   const int64_t stride = tb.stride;
   const int m = tb.nd_norb, nr = it.nr, nc = it.nc, pitch = (nc + 3) & ~3;
   g += (int64_t)it.r0 * stride + it.c0p;
@@ -436,16 +466,16 @@ __global__ void __launch_bounds__(Shape<G, SHAPE>::NT, Shape<G, SHAPE>::CTAS)
 }
 
 template <int G, int SHAPE>
-ed_status launch_one(const HvLaunch<float> *a, int64_t first, int64_t n, int mode,
-                     cudaStream_t st) {
+ed_status launch_one(const HvLaunch<float> *a, int mode, cudaStream_t st) {
+  const int64_t n = a ? a->tb.fib_n[SHAPE] : 0;
   if constexpr ((fiber_shapes(G) >> SHAPE) & 1) {
     constexpr int smem = 2 * Shape<G, SHAPE>::CAP * (int)sizeof(float);
     if (!a) {  // opt into large shared memory
       ED_TRY_CUDA(cudaFuncSetAttribute(k_hv_fiber<G, SHAPE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     } else if (n > 0) {
-      k_hv_fiber<G, SHAPE><<<(unsigned)n, Shape<G, SHAPE>::NT, smem, st>>>(*a, first,
-                                                                       mode == HV_LANCZOS);
+      k_hv_fiber<G, SHAPE><<<(unsigned)n, Shape<G, SHAPE>::NT, smem, st>>>(
+          *a, mode == HV_LANCZOS);
       ED_LAUNCHED(1);
     }
     return ED_OK;
@@ -458,10 +488,8 @@ ed_status launch_one(const HvLaunch<float> *a, int64_t first, int64_t n, int mod
 template <int G>
 ed_status launch_g(const HvLaunch<float> *a, int mode, cudaStream_t st) {
   if (a && mode != HV_PLAIN && mode != HV_LANCZOS) return ED_ERR_ARG;
-  int64_t f[FIBER_SHAPES + 1] = {0};
-  for (int s = 0; s < FIBER_SHAPES; ++s) f[s + 1] = f[s] + (a ? a->tb.fiber_n[s] : 0);
-  ED_TRY((launch_one<G, 0>(a, f[0], f[1] - f[0], mode, st)));
-  return launch_one<G, 1>(a, f[1], f[2] - f[1], mode, st);
+  ED_TRY((launch_one<G, 0>(a, mode, st)));
+  return launch_one<G, 1>(a, mode, st);
 }
 
 }  // namespace fiber

@@ -121,9 +121,7 @@ struct BlockInfo {
 struct HvItem {
   int32_t r0, nr, c0, nc;  // rows [r0, r0+nr) x columns [c0, c0+nc), one block pair
   int32_t c0p;             // first column in the vector layout (padded in block-major)
-  int32_t deg;             // ELL width of the up block (block-major), 0: use CSR;
-                           // orbital-factorised product: its group occupations, 4 bits
-                           // each, and the CTA shape from bit 24
+  int32_t deg;             // ELL width of the up block (block-major), 0: use CSR
   int32_t ell_off;         // first ELL entry of the up block
   int32_t ncp;             // ELL row length (padded block width)
 };
@@ -135,12 +133,22 @@ struct DwItem {
   int32_t r0, nr, c0p, nc;
 };
 
+// Up block of the orbital-factorised product: its columns, group occupations
+// (4 bits each), the rows of an item and the number of the block's first item
+// in its CTA shape's launch.  Item first + q covers rows q * rows .. of the
+// whole dw axis (the H_up pass does not mix rows).
+struct FibBlock {
+  int32_t c0, nc, c0p, keys, rows, first;
+};
+
 struct ItemList {
   HvItem *d_items = nullptr;
   int64_t nitems = 0;
   size_t smem = 0;
   int fiber = 0;               // group size of the orbital-factorised product, 0: not used
-  int64_t fiber_n[2] = {0, 0};  // its items per CTA shape (the list is in that order)
+  std::vector<FibBlock> fib;   // its up blocks, those of the first CTA shape first
+  FibBlock *d_fib = nullptr;
+  int nfib[2] = {0, 0};        // up blocks per CTA shape
   DwItem *d_ditems = nullptr;  // non-null: two-pass product (block pairs larger than L2)
   int64_t nditems = 0;
 };
@@ -321,10 +329,14 @@ struct HvTables {
   int64_t small_grid;      // its CTAs (= block partials of the Lanczos mode)
   int32_t small_chunk;     // its elements per thread
   bool passa_wide;         // two-pass product: the wide shape of the H_up pass
-  // orbital-factorised product (fiber.cuh): group size, 0 where not used; items
-  // per CTA shape; hop amplitudes of orbital k at hop_up[k (G - 1) + level]
+  // orbital-factorised product (fiber.cuh): group size, 0 where not used; per CTA
+  // shape the up blocks, the number of the first item and the items; the rows;
+  // hop amplitudes of orbital k at hop_up[k (G - 1) + level]
   int fiber = 0;
-  int64_t fiber_n[2] = {0, 0};
+  const FibBlock *fib[2] = {nullptr, nullptr};
+  int nfib[2] = {0, 0};
+  int64_t fib_first[2] = {0, 0}, fib_n[2] = {0, 0};
+  int64_t row0 = 0, rows = 0;
   T hop_up[ED_MAX_NS];
   // H_nd (spin exchange, pair hopping): move tables of this layout, or null
   const int32_t *nd_up = nullptr, *nd_dw = nullptr;

@@ -219,7 +219,14 @@ HvTables<float> ed_hv_tables<float>(ed_sector s, int layout) {
   t.small_chunk = (int32_t)small_chunk_of(s->bdim);
   t.passa_wide = layout == 1 && passa_is_wide(s);
   t.fiber = il.fiber;
-  for (int k = 0; k < FIBER_SHAPES; ++k) t.fiber_n[k] = il.fiber_n[k];
+  t.rows = s->sp[1].dim;
+  for (int k = 0, b = 0; k < FIBER_SHAPES; b += il.nfib[k], ++k) {
+    t.fib[k] = il.d_fib + b;
+    t.nfib[k] = il.nfib[k];
+    t.fib_n[k] = 0;
+    for (int q = b; q < b + il.nfib[k]; ++q)
+      t.fib_n[k] += (t.rows + il.fib[q].rows - 1) / il.fib[q].rows;
+  }
   for (int l = 0; l + s->mp.norb < s->mp.ns; ++l) t.hop_up[l] = (float)s->mp.V[0][s->mp.norb + l];
   set_nd<float>(t, s, layout);
   return t;
@@ -658,7 +665,28 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
   const int fiber = layout == 1 && elem == 4 ? fiber_group(s) : 0;
   std::vector<HvItem> items;
   size_t smem = 0;
-  for (size_t bd = 0; bd + 1 < ob_dw.size(); ++bd) {
+  std::vector<FibBlock> fib;
+  int nfib[2] = {0, 0};
+  if (fiber) {
+    // blocks by CTA shape; rows and items as fiber.cuh documents
+    const int64_t ddw = s->sp[1].dim;
+    for (int k = 0; k < FIBER_SHAPES; ++k) {
+      int64_t first = 0;
+      for (size_t bu = 0; bu + 1 < ob_up.size(); ++bu) {
+        const int64_t nc = ob_up[bu + 1] - ob_up[bu], pitch = round_up(nc, 4);
+        if (nc <= 0 || fiber_shape(fiber, pitch) != k) continue;
+        const int64_t R = std::min<int64_t>(FIBER_CAP[k] / pitch, FIBER_ROWS);
+        int32_t keys = 0;
+        for (int a = 0; a < s->mp.norb; ++a)
+          keys |= (int32_t)s->bi[0].keys[bu * s->mp.norb + a] << (4 * a);
+        fib.push_back(FibBlock{(int32_t)ob_up[bu], (int32_t)nc, (int32_t)op_up[bu], keys,
+                               (int32_t)R, (int32_t)first});
+        first += (ddw + R - 1) / R;
+        ++nfib[k];
+      }
+    }
+  }
+  for (size_t bd = 0; !fiber && bd + 1 < ob_dw.size(); ++bd) {
     const int64_t R0 = ob_dw[bd], R1 = ob_dw[bd + 1];
     if (R1 <= R0) continue;
     for (size_t bu = 0; bu + 1 < ob_up.size(); ++bu) {
@@ -674,26 +702,13 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
       R = std::min<int64_t>(std::min<int64_t>(R, HV_MAXROWS), R1 - R0);
       const size_t need = (size_t)((R + RT - 1) / RT) * per_group;
       if (need <= HV_SMEM_MAX) smem = std::max(smem, need);
-      int32_t deg = layout == 0 ? 0 : s->ell_deg[bu];
-      if (fiber) {
-        const int64_t pitch = round_up(nc, 4);
-        const int shape = fiber_shape(fiber, pitch);
-        R = std::min<int64_t>(std::min<int64_t>(FIBER_CAP[shape] / pitch, FIBER_ROWS), R1 - R0);
-        deg = shape << 24;
-        for (int k = 0; k < s->mp.norb; ++k)
-          deg |= (int32_t)s->bi[0].keys[bu * s->mp.norb + k] << (4 * k);
-      }
+      const int32_t deg = layout == 0 ? 0 : s->ell_deg[bu];
       const int32_t eoff = layout == 0 ? 0 : s->ell_off[bu];
       const int32_t ncp = (int32_t)(op_up[bu + 1] - op_up[bu]);
       for (int64_t r = R0; r < R1; r += R)
         items.push_back(HvItem{(int32_t)r, (int32_t)std::min<int64_t>(R, R1 - r), (int32_t)C0,
                                (int32_t)nc, (int32_t)op_up[bu], deg, eoff, ncp});
     }
-  }
-  if (fiber) {
-    std::stable_sort(items.begin(), items.end(),
-                     [](const HvItem &x, const HvItem &y) { return x.deg >> 24 < y.deg >> 24; });
-    for (const HvItem &x : items) ++il.fiber_n[x.deg >> 24];
   }
   HvItem *d_items = nullptr;
   ED_TRY(ed_dmalloc((void **)&d_items, std::max<size_t>(items.size(), 1) * sizeof(HvItem), cs,
@@ -702,16 +717,29 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
   if (!items.empty())
     e = cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(HvItem),
                         cudaMemcpyHostToDevice, cs);
+  FibBlock *d_fib = nullptr;
+  if (!fib.empty() && e == cudaSuccess) {
+    const ed_status fs = ed_dmalloc((void **)&d_fib, fib.size() * sizeof(FibBlock), cs, "work items");
+    if (fs != ED_OK) {
+      ed_dfree(d_items, cs);
+      return fs;
+    }
+    e = cudaMemcpyAsync(d_fib, fib.data(), fib.size() * sizeof(FibBlock), cudaMemcpyHostToDevice, cs);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
   if (e != cudaSuccess) {
     ed_set_cuda_error(e, "work items upload", __FILE__, __LINE__);
     ed_dfree(d_items, cs);
+    ed_dfree(d_fib, cs);
     return ED_ERR_CUDA;
   }
   // published only once complete
   il.nitems = (int64_t)items.size();
   il.smem = smem;
   il.fiber = fiber;
+  il.fib = fib;
+  il.d_fib = d_fib;
+  for (int k = 0; k < FIBER_SHAPES; ++k) il.nfib[k] = nfib[k];
   il.d_items = d_items;
   s->device_bytes += (int64_t)(items.size() * sizeof(HvItem));
   if (layout == 1) {
@@ -1410,7 +1438,7 @@ ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v,
   const int64_t np = tb.small_cols ? tb.small_grid
                                    : (tb.ditems ? tb.nditems : tb.nitems);
   if (nparts) *nparts = np;
-  if (tb.nitems == 0 || tb.dup == 0) return ED_OK;
+  if ((tb.fiber ? tb.rows : tb.nitems) == 0 || tb.dup == 0) return ED_OK;
   if (!tb.items) return ED_ERR_ARG;
   a.v = v;
   a.w = w;

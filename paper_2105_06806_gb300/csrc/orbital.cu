@@ -131,9 +131,21 @@ ed_status view_tables(ed_sector s, const OrbView &v, Mem &store, HvTables<T> *tb
   *tb = ed_hv_tables<T>(s, 1);
   tb->items = d_items;
   tb->nitems = (int64_t)keep.size();
-  if (tb->fiber) {
-    for (int64_t &n : tb->fiber_n) n = 0;
-    for (const HvItem &it : keep) ++tb->fiber_n[it.deg >> 24];
+  if (tb->fiber) {  // the block's descriptor over the block pair's rows
+    tb->row0 = v.R0;
+    tb->rows = v.nr;
+    for (int k = 0, q = 0; k < FIBER_SHAPES; ++k) {
+      const int n = il.nfib[k];
+      tb->fib_n[k] = tb->nfib[k] = 0;
+      for (const int end = q + n; q < end; ++q) {
+        const FibBlock &b = il.fib[q];
+        if (b.c0 != v.C0) continue;
+        tb->fib[k] = il.d_fib + q;
+        tb->nfib[k] = 1;
+        tb->fib_first[k] = b.first;
+        tb->fib_n[k] = (v.nr + b.rows - 1) / b.rows;
+      }
+    }
   }
   tb->ditems = il.d_ditems ? d_ditems : nullptr;
   tb->nditems = il.d_ditems ? (int64_t)dkeep.size() : 0;

@@ -398,6 +398,7 @@ static void sector_destroy(ed_sector s, cudaStream_t st) {
     for (int e = 0; e < 2; ++e) {
       ed_dfree(s->items[sp][e].d_items, st);
       ed_dfree(s->items[sp][e].d_ditems, st);
+      ed_dfree(s->items[sp][e].d_fib, st);
     }
   }
   ed_dfree(s->colpos, st);
