@@ -47,34 +47,62 @@ bool make_params(const ed_sector s, const ed_phonon *ph, PhParams *out) {
   return true;
 }
 
+// E consecutive elements as 16-byte vectors (E = 4) or one by one (E = 1).
+template <typename T, int E>
+struct alignas(E == 4 ? 16 : sizeof(T)) PhVec {
+  T x[E];
+};
+
 // w[p][i] += w0 p v[p][i] + N_g(i) (sqrt(p) v[p-1][i] + sqrt(p+1) v[p+1][i])
-// for every electronic element i of a slice (padding columns skipped).
-// Layout: element i = r * stride + c; the up mask of column c is
-// mup[padinv ? padinv[c] : c] (padinv < 0: padding), the dw mask mdw[r].
-template <typename T>
-__global__ void __launch_bounds__(PH_THREADS) k_phonon(const T *v, T *w, int64_t slice,
+// for every electronic element i of a slice (padding columns keep their
+// value).  Layout: element i = r * stride + c; the up mask of column c is
+// mup[padinv ? padinv[c] : c] (padinv < 0: padding), the dw mask mdw[r].  A
+// thread walks E elements' slices with a three-value window; the loads of the
+// next slice's v and w are issued before this slice's store.  E = 4 (slices
+// and rows of 4 k elements, 16-byte aligned): 16-byte accesses.
+template <typename T, int E>
+__global__ void __launch_bounds__(PH_THREADS) k_phonon(const T *__restrict__ v, T *w, int64_t slice,
                                                        int64_t stride, const int32_t *padinv,
                                                        const uint8_t *mup, const uint8_t *mdw,
                                                        PhParams ph) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < slice;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / stride, c = i - r * stride;
-    int64_t cu = c;
-    if (padinv) {
-      cu = padinv[c];
-      if (cu < 0) continue;
+  using V = PhVec<T, E>;
+  const int64_t n = slice / E;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
+       q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = q * E, r = i / stride, c = i - r * stride;
+    const double gd = ph.gm[mdw[r]];
+    T ng[E];
+    bool real[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int64_t cu = padinv ? (int64_t)padinv[c + e] : c + e;
+      real[e] = cu >= 0;
+      ng[e] = real[e] ? (T)(ph.gm[mup[cu]] + gd) : T(0);
     }
-    const T ng = (T)(ph.gm[mup[cu]] + ph.gm[mdw[r]]);
     const T w0 = (T)ph.w0;
-    T xm = T(0), x0 = v[i];
+    V xm, x0, o;
+#pragma unroll
+    for (int e = 0; e < E; ++e) xm.x[e] = T(0);
+    x0 = *reinterpret_cast<const V *>(v + i);
+    o = *reinterpret_cast<const V *>(w + i);
     for (int p = 0; p <= ph.nph; ++p) {
-      const T xp = p < ph.nph ? v[(int64_t)(p + 1) * slice + i] : T(0);
+      V xp, on;
+#pragma unroll
+      for (int e = 0; e < E; ++e) xp.x[e] = on.x[e] = T(0);
+      if (p < ph.nph) {
+        xp = *reinterpret_cast<const V *>(v + (int64_t)(p + 1) * slice + i);
+        on = *reinterpret_cast<const V *>(w + (int64_t)(p + 1) * slice + i);
+      }
       const T sp = sqrt((T)p), sp1 = sqrt((T)(p + 1));
-      const T disp = sp * xm + sp1 * xp;
-      T *o = w + (int64_t)p * slice + i;
-      *o = *o + (w0 * (T)p * x0 + ng * disp);
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const T disp = sp * xm.x[e] + sp1 * xp.x[e];
+        if (real[e]) o.x[e] = o.x[e] + (w0 * (T)p * x0.x[e] + ng[e] * disp);
+      }
+      *reinterpret_cast<V *>(w + (int64_t)p * slice + i) = o;
       xm = x0;
       x0 = xp;
+      o = on;
     }
   }
 }
@@ -115,15 +143,31 @@ unsigned grid_of(int64_t n) {
 template <typename T>
 ed_status eph_apply(ed_sector s, const PhParams &ph, int layout, const T *v, T *w,
                     cudaStream_t cs, const HvTables<T> *tables = nullptr) {
-  const HvTables<T> tb = tables ? *tables : ed_hv_tables<T>(s, layout);
+  HvTables<T> tb = tables ? *tables : ed_hv_tables<T>(s, layout);
   const int64_t slice = layout == 1 ? s->bdim : s->dim;
-  for (int p = 0; p <= ph.nph; ++p)
-    ED_TRY(ed_launch_hv<T>(s, tb, HV_PLAIN, v + (int64_t)p * slice, w + (int64_t)p * slice,
-                           nullptr, nullptr, nullptr, nullptr, nullptr, cs));
+  // the sector's kernel was chosen on one slice: with all slices in a launch
+  // the FP32 tiled family has the work to fill the GPU and is the faster one
+  // (the same w bit for bit)
+  if (sizeof(T) == 4 && slice * (ph.nph + 1) >= (int64_t)1 << 22) tb.small_cols = nullptr;
+  // every slice in one launch: a slice of a small sector does not fill the GPU.
+  // Bound: the product's shared-memory gathers (62 us), then k_phonon on
+  // L2-resident slices (15 us, 7.4 TB/s).  Norb=1 Ns=12, 11 slices, FP32: 85 us
+  // against 223 us with a launch per slice on CSR rows and an element per
+  // thread in k_phonon.
+  ED_TRY(ed_launch_hv<T>(s, tb, HV_PLAIN, v, w, nullptr, nullptr, nullptr, nullptr, nullptr, cs,
+                         nullptr, ph.nph + 1, slice));
   const SpinTables *t = layout == 1 ? s->bk : s->sp;
-  k_phonon<T><<<grid_of(slice), PH_THREADS, 0, cs>>>(v, w, slice, tb.stride,
-                                                     layout == 1 ? s->padinv : nullptr, t[0].imask,
-                                                     t[1].imask, ph);
+  const bool vec = slice % 4 == 0 && tb.stride % 4 == 0 &&
+                   (((uintptr_t)v | (uintptr_t)w) & 15) == 0;
+  const unsigned grid = (unsigned)std::max<int64_t>(
+      1, std::min<int64_t>((slice / (vec ? 4 : 1) + PH_THREADS - 1) / PH_THREADS, 1 << 20));
+  const int32_t *padinv = layout == 1 ? s->padinv : nullptr;
+  if (vec)
+    k_phonon<T, 4><<<grid, PH_THREADS, 0, cs>>>(v, w, slice, tb.stride, padinv, t[0].imask,
+                                                t[1].imask, ph);
+  else
+    k_phonon<T, 1><<<grid, PH_THREADS, 0, cs>>>(v, w, slice, tb.stride, padinv, t[0].imask,
+                                                t[1].imask, ph);
   ED_LAUNCHED(1);
   return ED_OK;
 }
@@ -197,13 +241,15 @@ extern "C" ed_status ed_eph_matvec(ed_sector s, const ed_phonon *ph, ed_precisio
     return ED_ERR_ARG;
   }
   cudaStream_t cs = (cudaStream_t)stream;
+  // sector-order slices that are block-major as they are (see matvec_layout)
+  const int layout = ed_same_layout(s) && (((uintptr_t)d_v | (uintptr_t)d_w) & 15) == 0 ? 1 : 0;
   if (prec == ED_FP64) {
-    ED_TRY(ed_build_items(s, 0, 8));
-    return eph_apply<double>(s, pp, 0, (const double *)d_v, (double *)d_w, cs);
+    ED_TRY(ed_build_items(s, layout, 8));
+    return eph_apply<double>(s, pp, layout, (const double *)d_v, (double *)d_w, cs);
   }
   if (prec == ED_FP32 || prec == ED_FP32_POLISH) {
-    ED_TRY(ed_build_items(s, 0, 4));
-    return eph_apply<float>(s, pp, 0, (const float *)d_v, (float *)d_w, cs);
+    ED_TRY(ed_build_items(s, layout, 4));
+    return eph_apply<float>(s, pp, layout, (const float *)d_v, (float *)d_w, cs);
   }
   return ED_ERR_ARG;
 }

@@ -347,8 +347,8 @@ __global__ void __launch_bounds__(Shape<G, SHAPE>::NT, Shape<G, SHAPE>::CTAS)
   __shared__ uint8_t s_md[FIBER_ROWS];
   __shared__ FibItem s_it;
   const HvTables<float> &tb = a.tb;
-  const float *g = a.v;
-  float *out = a.w;
+  const float *g = a.v + blockIdx.y * a.slice;
+  float *out = a.w + blockIdx.y * a.slice;
   if (lanczos) {
     const LanczosState *st = a.st;
     if (st->done) return;
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(Shape<G, SHAPE>::NT, Shape<G, SHAPE>::CTAS)
 }
 
 template <int G, int SHAPE>
-ed_status launch_one(const HvLaunch<float> *a, int mode, cudaStream_t st) {
+ed_status launch_one(const HvLaunch<float> *a, int mode, unsigned ns, cudaStream_t st) {
   const int64_t n = a ? a->tb.fib_n[SHAPE] : 0;
   if constexpr ((fiber_shapes(G) >> SHAPE) & 1) {
     constexpr int smem = 2 * Shape<G, SHAPE>::CAP * (int)sizeof(float);
@@ -474,7 +474,7 @@ ed_status launch_one(const HvLaunch<float> *a, int mode, cudaStream_t st) {
       ED_TRY_CUDA(cudaFuncSetAttribute(k_hv_fiber<G, SHAPE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     } else if (n > 0) {
-      k_hv_fiber<G, SHAPE><<<(unsigned)n, Shape<G, SHAPE>::NT, smem, st>>>(
+      k_hv_fiber<G, SHAPE><<<dim3((unsigned)n, ns), Shape<G, SHAPE>::NT, smem, st>>>(
           *a, mode == HV_LANCZOS);
       ED_LAUNCHED(1);
     }
@@ -486,10 +486,10 @@ ed_status launch_one(const HvLaunch<float> *a, int mode, cudaStream_t st) {
 // One launch per shape that the sector's items need; a == nullptr: prepares
 // the kernels of this G on the current device.
 template <int G>
-ed_status launch_g(const HvLaunch<float> *a, int mode, cudaStream_t st) {
+ed_status launch_g(const HvLaunch<float> *a, int mode, unsigned ns, cudaStream_t st) {
   if (a && mode != HV_PLAIN && mode != HV_LANCZOS) return ED_ERR_ARG;
-  ED_TRY((launch_one<G, 0>(a, mode, st)));
-  return launch_one<G, 1>(a, mode, st);
+  ED_TRY((launch_one<G, 0>(a, mode, ns, st)));
+  return launch_one<G, 1>(a, mode, ns, st);
 }
 
 }  // namespace fiber

@@ -3,5 +3,5 @@
 #include "fiber.cuh"
 
 namespace fiber {
-template ed_status launch_g<7>(const HvLaunch<float> *, int, cudaStream_t);
+template ed_status launch_g<7>(const HvLaunch<float> *, int, unsigned, cudaStream_t);
 }  // namespace fiber

@@ -3,8 +3,8 @@
 #include "fiber.cuh"
 
 namespace fiber {
-template ed_status launch_g<2>(const HvLaunch<float> *, int, cudaStream_t);
-template ed_status launch_g<3>(const HvLaunch<float> *, int, cudaStream_t);
-template ed_status launch_g<4>(const HvLaunch<float> *, int, cudaStream_t);
-template ed_status launch_g<5>(const HvLaunch<float> *, int, cudaStream_t);
+template ed_status launch_g<2>(const HvLaunch<float> *, int, unsigned, cudaStream_t);
+template ed_status launch_g<3>(const HvLaunch<float> *, int, unsigned, cudaStream_t);
+template ed_status launch_g<4>(const HvLaunch<float> *, int, unsigned, cudaStream_t);
+template ed_status launch_g<5>(const HvLaunch<float> *, int, unsigned, cudaStream_t);
 }  // namespace fiber

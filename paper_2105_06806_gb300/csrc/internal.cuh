@@ -442,7 +442,10 @@ template <typename T>
 ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v, T *w,
                        T *const *bufs, T *psi, LanczosState *state, double *part,
                        int64_t *nparts, cudaStream_t st,
-                       T *const *basis = nullptr);
+                       T *const *basis = nullptr, int nslices = 1, int64_t slice = 0);
+// True when vectors in sector order are block-major vectors as they are: one
+// orbital (the two orders agree) with no padding columns.
+inline bool ed_same_layout(ed_sector s) { return s->mp.norb == 1 && s->bstride == s->sp[0].dim; }
 
 int64_t ed_hv_num_parts(ed_sector s, int layout, int elem_size);
 template <typename T>

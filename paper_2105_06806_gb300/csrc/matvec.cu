@@ -132,17 +132,18 @@ static bool passa_is_wide(ed_sector s);
 // fiber.cuh: launch of the orbital-factorised product (a = nullptr: prepare)
 namespace fiber {
 template <int G>
-ed_status launch_g(const HvLaunch<float> *a, int mode, cudaStream_t st);
+ed_status launch_g(const HvLaunch<float> *a, int mode, unsigned ns, cudaStream_t st);
 }
-static ed_status launch_fiber(int g, const HvLaunch<float> *a, int mode, cudaStream_t st) {
+static ed_status launch_fiber(int g, const HvLaunch<float> *a, int mode, unsigned ns,
+                              cudaStream_t st) {
   switch (g) {
-    case 2: return fiber::launch_g<2>(a, mode, st);
-    case 3: return fiber::launch_g<3>(a, mode, st);
-    case 4: return fiber::launch_g<4>(a, mode, st);
-    case 5: return fiber::launch_g<5>(a, mode, st);
-    case 6: return fiber::launch_g<6>(a, mode, st);
-    case 7: return fiber::launch_g<7>(a, mode, st);
-    case 8: return fiber::launch_g<8>(a, mode, st);
+    case 2: return fiber::launch_g<2>(a, mode, ns, st);
+    case 3: return fiber::launch_g<3>(a, mode, ns, st);
+    case 4: return fiber::launch_g<4>(a, mode, ns, st);
+    case 5: return fiber::launch_g<5>(a, mode, ns, st);
+    case 6: return fiber::launch_g<6>(a, mode, ns, st);
+    case 7: return fiber::launch_g<7>(a, mode, ns, st);
+    case 8: return fiber::launch_g<8>(a, mode, ns, st);
   }
   return ED_ERR_ARG;
 }
@@ -907,8 +908,8 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
   const T *g;
   T *out_plain = nullptr;
   if (MODE == HV_PLAIN) {
-    g = a.v;
-    out_plain = a.w;
+    g = a.v + blockIdx.y * a.slice;
+    out_plain = a.w + blockIdx.y * a.slice;
   } else {
     const LanczosState *st = a.st;
     if (MODE == HV_LANCZOS && st->done) return;
@@ -1144,8 +1145,8 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
   const T *prev = nullptr;
   T *out;
   if (MODE == HV_PLAIN) {
-    g = a.v;
-    out = a.w;
+    g = a.v + blockIdx.y * a.slice;
+    out = a.w + blockIdx.y * a.slice;
   } else {
     const LanczosState *st = a.st;
     if (MODE == HV_LANCZOS && st->done) return;
@@ -1265,8 +1266,8 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
   const T *prev = nullptr;
   T *out;
   if (MODE == HV_PLAIN) {
-    g = a.v;
-    out = a.w;
+    g = a.v + blockIdx.y * a.slice;
+    out = a.w + blockIdx.y * a.slice;
   } else {
     const LanczosState *st = a.st;
     if (MODE == HV_LANCZOS && st->done) return;
@@ -1390,7 +1391,7 @@ ed_status ed_hv_prepare() {
   ED_TRY((prepare_layout<T, false>()));
   ED_TRY((prepare_layout<T, true>()));
   if (sizeof(T) == 4)
-    for (int g = FIBER_MIN_G; g <= FIBER_MAX_G; ++g) ED_TRY(launch_fiber(g, nullptr, 0, nullptr));
+    for (int g = FIBER_MIN_G; g <= FIBER_MAX_G; ++g) ED_TRY(launch_fiber(g, nullptr, 0, 1, nullptr));
   if (dev < 64) done[dev] = true;
   return ED_OK;
 }
@@ -1398,30 +1399,30 @@ template ed_status ed_hv_prepare<float>();
 template ed_status ed_hv_prepare<double>();
 
 template <typename T, int MODE>
-static ed_status launch_mode(const HvLaunch<T> &a, cudaStream_t st) {
+static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st) {
   if (a.tb.small_cols) {
     if (a.tb.small_chunk > 1)
-      k_hv_small<T, MODE, true><<<(unsigned)a.tb.small_grid, HVS_THREADS, 0, st>>>(a);
+      k_hv_small<T, MODE, true><<<dim3((unsigned)a.tb.small_grid, ns), HVS_THREADS, 0, st>>>(a);
     else
-      k_hv_small<T, MODE, false><<<(unsigned)a.tb.small_grid, HVS_THREADS, 0, st>>>(a);
+      k_hv_small<T, MODE, false><<<dim3((unsigned)a.tb.small_grid, ns), HVS_THREADS, 0, st>>>(a);
   } else if (a.tb.fiber) {
     if constexpr (sizeof(T) == 4) {
-      ED_TRY(launch_fiber(a.tb.fiber, &a, MODE, st));
+      ED_TRY(launch_fiber(a.tb.fiber, &a, MODE, ns, st));
     }
-    k_hv_dw<T, MODE><<<(unsigned)a.tb.nditems, DW_THREADS, 0, st>>>(a);
+    k_hv_dw<T, MODE><<<dim3((unsigned)a.tb.nditems, ns), DW_THREADS, 0, st>>>(a);
   } else if (a.tb.ditems) {
     if (a.tb.passa_wide)
       k_hv<T, MODE, true, true, rt_passa<T, true>(), passa_threads<true>()>
-          <<<(unsigned)a.tb.nitems, passa_threads<true>(), a.tb.smem, st>>>(a);
+          <<<dim3((unsigned)a.tb.nitems, ns), passa_threads<true>(), a.tb.smem, st>>>(a);
     else
       k_hv<T, MODE, true, true, rt_passa<T, false>(), passa_threads<false>()>
-          <<<(unsigned)a.tb.nitems, passa_threads<false>(), a.tb.smem, st>>>(a);
+          <<<dim3((unsigned)a.tb.nitems, ns), passa_threads<false>(), a.tb.smem, st>>>(a);
     ED_LAUNCHED(1);
-    k_hv_dw<T, MODE><<<(unsigned)a.tb.nditems, DW_THREADS, 0, st>>>(a);
+    k_hv_dw<T, MODE><<<dim3((unsigned)a.tb.nditems, ns), DW_THREADS, 0, st>>>(a);
   } else if (a.tb.ell_col) {
-    k_hv<T, MODE, true><<<(unsigned)a.tb.nitems, HV_THREADS, a.tb.smem, st>>>(a);
+    k_hv<T, MODE, true><<<dim3((unsigned)a.tb.nitems, ns), HV_THREADS, a.tb.smem, st>>>(a);
   } else {
-    k_hv<T, MODE, false><<<(unsigned)a.tb.nitems, HV_THREADS, a.tb.smem, st>>>(a);
+    k_hv<T, MODE, false><<<dim3((unsigned)a.tb.nitems, ns), HV_THREADS, a.tb.smem, st>>>(a);
   }
   ED_LAUNCHED(1);
   return ED_OK;
@@ -1430,7 +1431,9 @@ static ed_status launch_mode(const HvLaunch<T> &a, cudaStream_t st) {
 template <typename T>
 ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v, T *w,
                        T *const *bufs, T *psi, LanczosState *state, double *part,
-                       int64_t *nparts, cudaStream_t st, T *const *basis) {
+                       int64_t *nparts, cudaStream_t st, T *const *basis, int nslices,
+                       int64_t slice) {
+  if (nslices < 1 || nslices > 65535 || (nslices > 1 && mode != HV_PLAIN)) return ED_ERR_ARG;
   ED_TRY(ed_hv_prepare<T>());
   HvLaunch<T> a;
   a.tb = tb;
@@ -1449,21 +1452,25 @@ ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v,
   a.psi = psi;
   a.st = state;
   a.part = part;
-  if (mode == HV_PLAIN) ED_TRY((launch_mode<T, HV_PLAIN>(a, st)));
-  else if (mode == HV_LANCZOS) ED_TRY((launch_mode<T, HV_LANCZOS>(a, st)));
-  else ED_TRY((launch_mode<T, HV_SECOND>(a, st)));
+  a.slice = slice;
+  if (mode == HV_PLAIN) ED_TRY((launch_mode<T, HV_PLAIN>(a, (unsigned)nslices, st)));
+  else if (mode == HV_LANCZOS) ED_TRY((launch_mode<T, HV_LANCZOS>(a, 1, st)));
+  else ED_TRY((launch_mode<T, HV_SECOND>(a, 1, st)));
   if (!tb.nd_up) return ED_OK;
   // spin exchange and pair hopping, added to the product (partials after the product's)
   if (nparts) *nparts = np + ed_nd_grid(tb.ddw, tb.nd_ncols);
+  for (int p = 1; p < nslices; ++p)
+    ED_TRY(ed_launch_nd<T>(tb, mode, v + p * slice, w + p * slice, bufs, basis, state, nullptr, st));
   return ed_launch_nd<T>(tb, mode, v, w, bufs, basis, state, part ? part + np : nullptr, st);
 }
 
 template ed_status ed_launch_hv<float>(ed_sector, const HvTables<float> &, int, const float *,
                                        float *, float *const *, float *, LanczosState *, double *,
-                                       int64_t *, cudaStream_t, float *const *);
+                                       int64_t *, cudaStream_t, float *const *, int, int64_t);
 template ed_status ed_launch_hv<double>(ed_sector, const HvTables<double> &, int, const double *,
                                         double *, double *const *, double *, LanczosState *,
-                                        double *, int64_t *, cudaStream_t, double *const *);
+                                        double *, int64_t *, cudaStream_t, double *const *, int,
+                                        int64_t);
 
 static ed_status matvec_layout(ed_sector s, ed_precision prec, const void *d_v, void *d_w,
                                int64_t n, void *stream, int layout) {
@@ -1480,6 +1487,9 @@ static ed_status matvec_layout(ed_sector s, ed_precision prec, const void *d_v, 
                                  : "vectors must be aligned to their element size");
     return ED_ERR_ARG;
   }
+  // sector-order vectors that are block-major as they are take that layout's
+  // kernels (ELL table and 16-byte accesses instead of CSR rows)
+  if (layout == 0 && ed_same_layout(s) && (((uintptr_t)d_v | (uintptr_t)d_w) & 15) == 0) layout = 1;
   cudaStream_t st = (cudaStream_t)stream;
   if (prec == ED_FP64) {
     ED_TRY(ed_build_items(s, layout, 8));

@@ -62,6 +62,7 @@ struct HvLaunch {
   T *psi;
   LanczosState *st;
   double *part;
+  int64_t slice = 0;  // HV_PLAIN: grid row y works on v + y * slice, w + y * slice
 };
 
 template <typename T>
