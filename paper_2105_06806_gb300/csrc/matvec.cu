@@ -901,7 +901,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
   struct EpState {
     T *out;
     const T *prev;
-    T s_cur, s_prev, beta_j, alpha_j, y_j;
+    T s_cur, beta_s, alpha_s, y_s;  // scale of v_j; beta, alpha, y times their vector's scale
     int j;
   };
   __shared__ EpState ep_s;
@@ -926,11 +926,11 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
         e.prev = a.basis[j > 0 ? j - 1 : 0];
         e.out = a.basis[j + 1];
       }
-      e.s_cur = (T)st->scale[j % 3];
-      e.s_prev = (T)st->scale[(j + 2) % 3];
-      e.beta_j = (T)st->beta[j];
-      e.alpha_j = MODE == HV_SECOND ? (T)st->alpha[j] : T(0);
-      e.y_j = MODE == HV_SECOND ? (T)st->y[j] : T(0);
+      const double sc = st->scale[j % 3];
+      e.s_cur = (T)sc;
+      e.beta_s = (T)(st->beta[j] * st->scale[(j + 2) % 3]);
+      e.alpha_s = MODE == HV_SECOND ? (T)(st->alpha[j] * sc) : T(0);
+      e.y_s = MODE == HV_SECOND ? (T)(st->y[j] * sc) : T(0);
       ep_s = e;
     }
   }
@@ -1051,7 +1051,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
               if (i >= nrt || (!full && c >= nc)) continue;
               const T w1 = mul_t<T>(acc[u][i], s_cur);
               acc[u][i] = w1;
-              dot = fma_t<T>(mul_t<T>(xr[i], s_cur), w1, dot);
+              dot = fma_t<T>(xr[i], w1, dot);
             }
           }
 #pragma unroll
@@ -1070,8 +1070,8 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
           continue;
         }
         // second pass: the step's scalars, read from shared memory once per tile
-        const T s_cur = ep.s_cur, s_prev = ep.s_prev, beta_j = ep.beta_j;
-        const T alpha_j = ep.alpha_j, y_j = ep.y_j;
+        const T s_cur = ep.s_cur, beta_s = ep.beta_s;
+        const T alpha_s = ep.alpha_s, y_s = ep.y_s;
         const T *const prev = ep.prev;
         const bool has_prev = ep.j > 0;
 #pragma unroll
@@ -1095,16 +1095,10 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
             res[u] = T(0);
             if (!full && c >= nc) continue;
             const T xv = staged ? smq[(size_t)stage_pos(c, ncp >> 2) * RT + i] : g[rb + u];
-            const T v = mul_t<T>(xv, s_cur);
             T w1 = mul_t<T>(acc[u][i], s_cur);
-            if (has_prev) w1 = fma_t<T>(-beta_j, mul_t<T>(pv[u], s_prev), w1);
-            if (MODE == HV_LANCZOS) {
-              res[u] = w1;
-              dot = fma_t<T>(v, w1, dot);
-            } else {
-              res[u] = fma_t<T>(-alpha_j, v, w1);
-              a.psi[rb + u] = fma_t<T>(y_j, v, a.psi[rb + u]);
-            }
+            if (has_prev) w1 = fma_t<T>(-beta_s, pv[u], w1);
+            res[u] = fma_t<T>(-alpha_s, xv, w1);
+            a.psi[rb + u] = fma_t<T>(y_s, xv, a.psi[rb + u]);
           }
           if (vec) {
             store4(out + rb, res);
@@ -1118,8 +1112,9 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
     }
   }
   if (MODE == HV_LANCZOS && !PASSA) {
+    // <v_j, w1> with v_j = s_cur * (the vector read)
     double smv = block_sum<T>((double)dot, red);
-    if (threadIdx.x == 0) a.part[blockIdx.x] = smv;
+    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * (double)ep_s.s_cur;
   }
 }
 
@@ -1134,13 +1129,13 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
 template <typename T, int MODE>
 __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
   constexpr int RT = Tile<T>::RT;
-  __shared__ double red[DW_THREADS / 32];
+  __shared__ double red[MODE == HV_LANCZOS ? DW_THREADS : 1];
   __shared__ int32_t s_dcol[DW_ROWS * ED_MAX_NS];
   __shared__ T s_dval[DW_ROWS * ED_MAX_NS];
   __shared__ int32_t s_dn[DW_ROWS];
   const HvTables<T> &tb = a.tb;
   int j = 0;
-  T s_cur = T(1), s_prev = T(0), beta_j = T(0), alpha_j = T(0), y_j = T(0);
+  T s_cur = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
   const T *g;
   const T *prev = nullptr;
   T *out;
@@ -1161,11 +1156,10 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
       out = a.basis[j + 1];
     }
     s_cur = (T)st->scale[m3];
-    s_prev = (T)st->scale[(j + 2) % 3];
-    beta_j = (T)st->beta[j];
     if (MODE == HV_SECOND) {
-      alpha_j = (T)st->alpha[j];
-      y_j = (T)st->y[j];
+      beta_s = (T)(st->beta[j] * st->scale[(j + 2) % 3]);
+      alpha_s = (T)(st->alpha[j] * st->scale[m3]);
+      y_s = (T)(st->y[j] * st->scale[m3]);
     }
   }
   const DwItem it = tb.ditems[blockIdx.x];
@@ -1230,24 +1224,24 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
         if (MODE == HV_PLAIN) {
           out[gi] = acc[i][u];
         } else {
-          const T v = mul_t<T>(g[gi], s_cur);
+          const T x = g[gi];
           T w1 = mul_t<T>(acc[i][u], s_cur);
           if (MODE == HV_SECOND && j > 0)  // the Lanczos step does this in its update
-            w1 = fma_t<T>(-beta_j, mul_t<T>(prev[gi], s_prev), w1);
+            w1 = fma_t<T>(-beta_s, prev[gi], w1);
           if (MODE == HV_LANCZOS) {
             out[gi] = w1;
-            dot = fma_t<T>(v, w1, dot);
+            dot = fma_t<T>(x, w1, dot);
           } else {
-            out[gi] = fma_t<T>(-alpha_j, v, w1);
-            a.psi[gi] = fma_t<T>(y_j, v, a.psi[gi]);
+            out[gi] = fma_t<T>(-alpha_s, x, w1);
+            a.psi[gi] = fma_t<T>(y_s, x, a.psi[gi]);
           }
         }
       }
     }
   }
   if (MODE == HV_LANCZOS) {
-    double smv = block_sum<T>(dotd + (double)dot, red);
-    if (threadIdx.x == 0) a.part[blockIdx.x] = smv;
+    const double smv = cta_sum<DW_THREADS>(dotd + (double)dot, red);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * (double)s_cur;  // v_j = s_cur x
   }
 }
 
@@ -1258,10 +1252,10 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
 // partial of <v_j, w1> per CTA.
 template <typename T, int MODE, bool CHUNKED>
 __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
-  __shared__ double red[HVS_THREADS / 32];
+  __shared__ double red[MODE == HV_LANCZOS ? HVS_THREADS : 1];
   const HvTables<T> &tb = a.tb;
   int j = 0;
-  T s_cur = T(1), s_prev = T(0), beta_j = T(0), alpha_j = T(0), y_j = T(0);
+  T s_cur = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
   const T *g;
   const T *prev = nullptr;
   T *out;
@@ -1281,12 +1275,11 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
       prev = a.basis[j > 0 ? j - 1 : 0];
       out = a.basis[j + 1];
     }
-    s_cur = (T)st->scale[j % 3];
-    s_prev = (T)st->scale[(j + 2) % 3];
-    beta_j = (T)st->beta[j];
+    s_cur = (T)st->scale[m3];
     if (MODE == HV_SECOND) {
-      alpha_j = (T)st->alpha[j];
-      y_j = (T)st->y[j];
+      beta_s = (T)(st->beta[j] * st->scale[(j + 2) % 3]);
+      alpha_s = (T)(st->alpha[j] * st->scale[m3]);
+      y_s = (T)(st->y[j] * st->scale[m3]);
     }
   }
   const int64_t stride = tb.stride;
@@ -1322,23 +1315,22 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
       if (MODE == HV_PLAIN) {
         out[gi] = acc;
       } else {
-        const T v = mul_t<T>(x, s_cur);
         T w1 = mul_t<T>(acc, s_cur);
         if (MODE == HV_SECOND && j > 0)  // the Lanczos step does this in its update
-          w1 = fma_t<T>(-beta_j, mul_t<T>(prev[gi], s_prev), w1);
+          w1 = fma_t<T>(-beta_s, prev[gi], w1);
         if (MODE == HV_LANCZOS) {
           out[gi] = w1;
-          dot = fma_t<T>(v, w1, dot);
+          dot = fma_t<T>(x, w1, dot);
         } else {
-          out[gi] = fma_t<T>(-alpha_j, v, w1);
-          a.psi[gi] = fma_t<T>(y_j, v, a.psi[gi]);
+          out[gi] = fma_t<T>(-alpha_s, x, w1);
+          a.psi[gi] = fma_t<T>(y_s, x, a.psi[gi]);
         }
       }
     }
   }
   if (MODE == HV_LANCZOS) {
-    double smv = block_sum<T>(dot_sum + (double)dot, red);
-    if (threadIdx.x == 0) a.part[blockIdx.x] = smv;
+    const double smv = cta_sum<HVS_THREADS>(dot_sum + (double)dot, red);
+    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * (double)s_cur;  // v_j = s_cur x
   }
 }
 

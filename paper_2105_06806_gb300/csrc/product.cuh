@@ -65,6 +65,26 @@ struct HvLaunch {
   int64_t slice = 0;  // HV_PLAIN: grid row y works on v + y * slice, w + y * slice
 };
 
+// Sum over a CTA of NT threads (fixed order), in thread 0 of the first warp:
+// the values cross shared memory and one warp adds them.  A shuffle tree in
+// every warp would cost each thread 5 FP64 additions, as much FP64 issue as a
+// third of an element's product (GB300 issues FP64 at 1/64 of the FP32 rate;
+// the FP64 Lanczos-mode product at 1.18e7 elements: 588 -> 474 us with this and
+// <v_j, w> summed before the scale of v_j is applied).
+template <int NT>
+__device__ __forceinline__ double cta_sum(double x, double *buf) {
+  buf[threadIdx.x] = x;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int k = 0; k < NT / 32; ++k) s += buf[threadIdx.x + 32 * k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  }
+  return s;
+}
+
 template <typename T>
 __device__ __forceinline__ double block_sum(double x, double *red) {
   for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
