@@ -550,7 +550,7 @@ ed_status ed_server_destroy(ed_server srv);
 /* Batched Green's-function launches of this process (no counterpart in the
  * paper; the task parallelism over independent impurity problems of Sec. 6.9
  * on one GPU).  The chains of solves whose N+-1 sectors are small (at most
- * 2^14 states) run in one persistent launch, one CTA per chain; solves that
+ * 2^14 states) run in one launch, a cluster of CTAs per chain; solves that
  * reach that phase at about the same time -- concurrent server requests,
  * or several host threads calling ed_solve -- share one launch (the first
  * one leads and waits at most 1 ms for the others).  A chain's result does

@@ -13,7 +13,11 @@
 #include <type_traits>
 #include <vector>
 
-#include "internal.cuh"
+#include <cooperative_groups.h>
+
+#include "product.cuh"
+
+namespace cg = cooperative_groups;
 
 constexpr int GF_THREADS = 256;
 
@@ -226,47 +230,54 @@ ed_status ed_cfrac_z_launch(const LanczosState *st, double weight, double e0, co
 
 // ----------------------------------------------------------------- batched chains
 //
-// All chains of a solve whose sectors are small run in one persistent launch:
-// each CTA takes a chain from a device counter and runs it to the end alone
-// (start vector c^+-|gs>, nsteps of the recurrence of lanczos.cu with the
-// element-parallel product, FP64 scalars), so a chain costs one CTA and no
-// host round trip.  The chains of a solve have different lengths (the
-// c^+ and c sectors differ in dimension); a CTA that finishes takes the next.
-// v_j is staged in shared memory every step, so every gather of the product
-// is a shared-memory load.
-constexpr int CHAIN_THREADS = 1024;
-// padded elements of a batched chain's sector (FP64: 128 KB of shared memory)
+// All chains of a solve whose sectors are small run in one launch: a cluster
+// of CHAIN_CTAS CTAs takes a chain and runs it to the end alone (start vector
+// c^+-|gs>, nsteps of the recurrence of lanczos.cu with the element-parallel
+// product, FP64 scalars), so a chain costs no host round trip.  Clusters take
+// the chains round robin.  Every CTA holds all of v_j in shared memory, so
+// every gather of the product is a shared-memory load, and forms 1 /
+// CHAIN_CTAS of the next vector, which it writes into every CTA's copy
+// through distributed shared memory; two cluster barriers per step (one per
+// inner product) order this.
+//
+// Bound: FP64 issue (17 operations per element and step in FP64; one SM has 2
+// FP64 lanes), then the two reductions and barriers.  One CTA per chain (the
+// first form of this kernel) took 5.74 ms for the two FP64 chains of 200
+// steps of an Ns=8 solve; a cluster of 8: 1.60 ms.  The cluster size is
+// fixed, so a chain's sums do not depend on the other chains of the launch.
+constexpr int CHAIN_THREADS = 256;
+constexpr int CHAIN_CTAS = 8;
+// padded elements of a batched chain's sector (FP64: 160 KB of shared memory)
 constexpr int64_t CHAIN_MAX_DIM = 1 << 14;
+// elements of shared memory for a sector of n: v_j, and a CTA's part of
+// v_{j-1} and of the new vector
+__host__ __device__ inline int64_t chain_part(int64_t n) { return (n + CHAIN_CTAS - 1) / CHAIN_CTAS; }
+__host__ __device__ inline int64_t chain_smem(int64_t n) { return n + 2 * chain_part(n); }
 
 template <typename Ti, typename To>
 struct ChainTask {
   HvTables<To> tb;     // target sector, block-major, element-parallel form
   ApplyArgs a;         // start vector gather
   const Ti *psi;       // ground state, sector order
-  To *b0, *b1, *b2;    // three vectors of a.dst_dim elements
   LanczosState *st;    // output: alpha, beta, j, acc[0] = ||phi||^2
   int nsteps;
 };
 
-// Sum over the CTA, the same value in every thread, fixed order, in FP64
-// (each thread's partial covers at most n / CHAIN_THREADS <= 16 elements of
-// a chain's sector, summed in the vector type).
-template <typename T>
-__device__ double chain_allsum(T xt, double *red) {
-  double x = (double)xt;
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = (double)x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
-    red[32] = t;
+// Sum over the cluster in thread 0 of every CTA (the same value: fixed order
+// in FP64, each thread's partial covers at most CHAIN_MAX_DIM / CHAIN_CTAS /
+// CHAIN_THREADS = 8 elements summed in the vector type).  Ends with a cluster
+// barrier passed; `slot` alternates between calls.
+__device__ double chain_sum(cg::cluster_group &cl, double x, double *red, double (&part)[2],
+                            int slot) {
+  const double s = cta_sum<CHAIN_THREADS>(x, red);
+  if (threadIdx.x == 0) part[slot] = s;
+  cl.sync();
+  double t = 0.0;
+  if (threadIdx.x < 32) {
+    if (threadIdx.x < CHAIN_CTAS) t = *cl.map_shared_rank(&part[slot], threadIdx.x);
+    for (int o = CHAIN_CTAS / 2; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
   }
-  __syncthreads();
-  const double r = red[32];
-  __syncthreads();
-  return r;
+  return t;
 }
 
 template <typename T>
@@ -277,35 +288,37 @@ template <>
 __device__ __forceinline__ double ch_fma<double>(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 template <typename Ti, typename To>
-__global__ void __launch_bounds__(CHAIN_THREADS) k_chain_batch(const ChainTask<Ti, To> *tasks,
-                                                               int ntasks, int *next) {
-  extern __shared__ __align__(16) unsigned char chain_smem[];
-  To *S = reinterpret_cast<To *>(chain_smem);  // v_j (unscaled) of the current step
-  __shared__ double red[33];
-  __shared__ double s_scal[2];
-  __shared__ int s_task, s_done;
-  for (;;) {
-    if (threadIdx.x == 0) s_task = atomicAdd(next, 1);
-    __syncthreads();
-    const int t = s_task;
-    __syncthreads();
-    if (t >= ntasks) return;
+__global__ void __cluster_dims__(CHAIN_CTAS, 1, 1) __launch_bounds__(CHAIN_THREADS)
+    k_chain_batch(const ChainTask<Ti, To> *tasks, int ntasks) {
+  extern __shared__ __align__(16) unsigned char chain_smem_raw[];
+  To *S = reinterpret_cast<To *>(chain_smem_raw);  // v_j (unscaled) of the current step
+  __shared__ double red[CHAIN_THREADS], part[2];
+  __shared__ double s_bc[4];  // scalars of thread 0 for the CTA
+  __shared__ int s_done;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  To *peer[CHAIN_CTAS];
+#pragma unroll
+  for (int q = 0; q < CHAIN_CTAS; ++q) peer[q] = cl.map_shared_rank(S, q);
+  for (int t = blockIdx.x / CHAIN_CTAS; t < ntasks; t += gridDim.x / CHAIN_CTAS) {
     const ChainTask<Ti, To> &tk = tasks[t];
     const HvTables<To> &tb = tk.tb;
     const ApplyArgs &a = tk.a;
-    const int64_t n = a.dst_dim, stride = a.dst_stride;
+    const int n = (int)a.dst_dim, stride = (int)a.dst_stride;
+    const int np = (int)chain_part(n), lo = rank * np, hi = min(n, lo + np);
+    To *P = S + n, *W = P + np;  // this CTA's part of v_{j-1} and of the new vector
     const float inv_stride = 1.0f / (float)stride;
-    To *bufs[3] = {tk.b0, tk.b1, tk.b2};
-    // start vector into b0 (the gather of k_apply_op), b1 = b2 = 0
+    cl.sync();  // the previous chain's vectors are no longer read
+    // start vector (the gather of k_apply_op)
     double sq = 0.0;
     {
       const uint32_t bit = 1u << a.level, below = bit - 1u;
-      for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+      for (int i = lo + threadIdx.x; i < hi; i += CHAIN_THREADS) {
         // exact row index: (i + 1/2) / stride lies 1/(2 stride) from an integer
-        const int64_t r2 = __float2int_rz(((float)i + 0.5f) * inv_stride);
+        const int r2 = __float2int_rz(((float)i + 0.5f) * inv_stride);
         const int32_t c2 = a.dst_padinv[i - r2 * stride];
         To out = To(0);
-        const uint32_t I2 = c2 < 0 ? 0u : a.dst_map[a.spin == 0 ? (int64_t)c2 : r2];
+        const uint32_t I2 = c2 < 0 ? 0u : a.dst_map[a.spin == 0 ? c2 : r2];
         if (c2 >= 0 && ((I2 & bit) != 0u) == (a.create > 0)) {
           const uint32_t I = I2 ^ bit;
           const int64_t src_idx = ed_rank(I);
@@ -316,36 +329,42 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_chain_batch(const ChainTask<T
           const Ti x = tk.psi[r * a.src_dup + c];
           out = (To)((parity & 1) ? -x : x);
         }
-        tk.b0[i] = out;
-        tk.b1[i] = To(0);
-        tk.b2[i] = To(0);
+#pragma unroll
+        for (int q = 0; q < CHAIN_CTAS; ++q) peer[q][i] = out;
+        P[i - lo] = To(0);
         sq += (double)out * (double)out;
       }
     }
-    const double weight = chain_allsum<double>(sq, red);
+    int slot = 0;
+    const double weight = chain_sum(cl, sq, red, part, slot);  // thread 0
+    slot ^= 1;
     LanczosState *st = tk.st;
-    double scale[3] = {weight > 0.0 ? 1.0 / sqrt(weight) : 0.0, 0.0, 0.0};
-    double beta_j = 0.0, tnorm = 0.0;
-    int j = 0, done = weight > 0.0 ? 0 : 2;
+    double tnorm = 0.0, scale = 0.0, scale_prev = 0.0;  // thread 0
     if (threadIdx.x == 0) {
-      st->acc[0] = weight;
-      st->beta[0] = 0.0;
+      if (rank == 0) {
+        st->acc[0] = weight;
+        st->beta[0] = 0.0;
+      }
+      scale = weight > 0.0 ? 1.0 / sqrt(weight) : 0.0;
+      s_bc[0] = scale;
+      s_bc[1] = 0.0;  // beta_j times the scale of v_{j-1}
+      s_done = weight > 0.0 ? 0 : 2;
     }
+    __syncthreads();
+    int j = 0, done = s_done;
+    double beta_j = 0.0;  // thread 0
     while (!done) {
-      const To *g = bufs[j % 3];
-      const To *prev = bufs[(j + 2) % 3];
-      To *out = bufs[(j + 1) % 3];
-      const To s_cur = (To)scale[j % 3], s_prev = (To)scale[(j + 2) % 3];
-      const To bj = (To)beta_j;
-      for (int64_t i = threadIdx.x; i < n; i += blockDim.x) S[i] = g[i];
-      __syncthreads();
+      const To s_cur = (To)s_bc[0], bs = (To)s_bc[1];
       // w1 = H v_j - beta_j v_{j-1} (padding columns are skipped: they stay 0)
-      To dot = To(0);  // per-thread partials in the vector type; FP64 across warps
-      for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const int64_t r = __float2int_rz(((float)i + 0.5f) * inv_stride);
-        const int pc = (int)(i - r * stride);
+      To dot = To(0);  // per-thread partials in the vector type; FP64 across threads
+      for (int i = lo + threadIdx.x; i < hi; i += CHAIN_THREADS) {
+        const int r = __float2int_rz(((float)i + 0.5f) * inv_stride);
+        const int pc = i - r * stride;
         const int4 ci = __ldg(tb.small_cols + pc);
-        if (ci.x < 0) continue;
+        if (ci.x < 0) {
+          W[i - lo] = To(0);
+          continue;
+        }
         const To x = S[i];
         const To *row = S + r * stride + ci.z;
         const int deg = ci.w & 255, ncp = ci.w >> 8;
@@ -357,48 +376,57 @@ __global__ void __launch_bounds__(CHAIN_THREADS) k_chain_batch(const ChainTask<T
         }
         const int32_t d0 = __ldg(tb.rp_dw + r), d1 = __ldg(tb.rp_dw + r + 1);
         for (int32_t k = d0; k < d1; ++k)
-          acc = ch_fma<To>(__ldg(tb.val_dw + k), S[(int64_t)__ldg(tb.col_dw + k) * stride + pc], acc);
+          acc = ch_fma<To>(__ldg(tb.val_dw + k), S[__ldg(tb.col_dw + k) * stride + pc], acc);
         if (tb.nd_up)  // spin exchange and pair hopping
           acc += ed_nd_terms<To>(tb, S, stride, r, pc, (int)tb.m_up[ci.x], (int)tb.m_dw[r]);
-        const To v = x * s_cur;
-        To w1 = acc * s_cur;
-        if (j > 0) w1 = ch_fma<To>(-bj, prev[i] * s_prev, w1);
-        out[i] = w1;
-        dot = ch_fma<To>(v, w1, dot);
+        const To w1 = ch_fma<To>(-bs, P[i - lo], acc * s_cur);
+        W[i - lo] = w1;
+        dot = ch_fma<To>(x, w1, dot);
       }
-      const double al = chain_allsum<To>(dot, red);
-      // w = w1 - alpha_j v_j, ||w||^2
-      const To alT = (To)al;
+      double al = chain_sum(cl, (double)dot, red, part, slot);
+      slot ^= 1;
+      if (threadIdx.x == 0) {
+        al *= scale;  // v_j = scale * S
+        s_bc[2] = al * scale;
+      }
+      __syncthreads();
+      // w = w1 - alpha_j v_j, ||w||^2; v_j becomes v_{j-1}
+      const To as = (To)s_bc[2];
       To ss = To(0);
-      for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const To w = ch_fma<To>(-alT, S[i] * s_cur, out[i]);
-        out[i] = w;
+      for (int i = lo + threadIdx.x; i < hi; i += CHAIN_THREADS) {
+        const To x = S[i];
+        const To w = ch_fma<To>(-as, x, W[i - lo]);
+        P[i - lo] = x;
+#pragma unroll
+        for (int q = 0; q < CHAIN_CTAS; ++q) peer[q][i] = w;
         ss = ch_fma<To>(w, w, ss);
       }
-      const double ss_tot = chain_allsum<To>(ss, red);
-      // scalar bookkeeping once, by thread 0
+      const double ss_tot = chain_sum(cl, (double)ss, red, part, slot);
+      slot ^= 1;
       if (threadIdx.x == 0) {
         const double be = sqrt(fmax(ss_tot, 0.0));
         tnorm = fmax(tnorm, fmax(fabs(al), be));
-        st->alpha[j] = al;
-        st->beta[j + 1] = be;
-        s_scal[0] = be;
-        s_scal[1] = be > 0.0 ? 1.0 / be : 0.0;
+        if (rank == 0) {
+          st->alpha[j] = al;
+          st->beta[j + 1] = be;
+        }
+        scale_prev = scale;
+        scale = be > 0.0 ? 1.0 / be : 0.0;
+        beta_j = be;
+        s_bc[0] = scale;
+        s_bc[1] = beta_j * scale_prev;
         s_done = be <= 1e-13 * tnorm ? 2 : (j + 1 >= tk.nsteps ? 3 : 0);
       }
       __syncthreads();
-      beta_j = s_scal[0];
-      scale[(j + 1) % 3] = s_scal[1];
       done = s_done;
       ++j;
-      __syncthreads();
     }
-    if (threadIdx.x == 0) {
+    if (rank == 0 && threadIdx.x == 0) {
       st->j = j;
       st->done = done;
     }
-    __syncthreads();
   }
+  cl.sync();  // no CTA leaves while a peer may still read its shared memory
 }
 
 // Continued fractions of a batch of chains (grid.y = chain): the arithmetic
@@ -644,7 +672,7 @@ bool ed_gf_batchable(ed_sector s, int spin, int create) {
 // caller of a (device, precision, grid) group leads it, waits a short window
 // for the others while other small solves are under way, then launches every
 // member's chains at once on its own stream after the members' streams.  A
-// chain runs on one CTA from its own task and workspace, so its coefficients
+// chain runs on one cluster from its own task and workspace, so its coefficients
 // and G do not depend on which other chains share the launch: a solve gives
 // the same result alone and in any mix.
 namespace {
@@ -716,9 +744,9 @@ ed_status run_group(const std::vector<BatchMember *> &ms, cudaStream_t cs) {
   const size_t o_sgn = o_sts + al256(nt * sizeof(LanczosState *));
   const size_t o_e0 = o_sgn + al256(nt * sizeof(int));
   const size_t o_G = o_e0 + al256(nt * sizeof(double));
-  const size_t o_next = o_G + al256((size_t)nt * std::max(nmats, 1) * sizeof(double2));
   void *mem = nullptr;
-  ED_TRY(ed_dmalloc(&mem, o_next + 256, cs, "batched chains"));
+  ED_TRY(ed_dmalloc(&mem, o_G + al256((size_t)nt * std::max(nmats, 1) * sizeof(double2)), cs,
+                    "batched chains"));
   char *base = (char *)mem;
   ed_status rs = ED_OK;
   for (const BatchMember *m : ms)
@@ -732,15 +760,15 @@ ed_status run_group(const std::vector<BatchMember *> &ms, cudaStream_t cs) {
   h2d(o_sts, sts.data(), nt * sizeof(LanczosState *));
   h2d(o_sgn, sgn.data(), nt * sizeof(int));
   h2d(o_e0, e0.data(), nt * sizeof(double));
-  if (rs == ED_OK && cudaMemsetAsync(base + o_next, 0, sizeof(int), cs) != cudaSuccess) rs = ED_ERR_CUDA;
   if (rs == ED_OK && cudaFuncSetAttribute(k_chain_batch<Ti, To>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)(CHAIN_MAX_DIM * sizeof(To))) != cudaSuccess)
+                                          (int)(chain_smem(CHAIN_MAX_DIM) * sizeof(To))) !=
+                         cudaSuccess)
     rs = ED_ERR_CUDA;
   if (rs == ED_OK) {
-    k_chain_batch<Ti, To><<<(unsigned)std::min(nt, 2 * 152), CHAIN_THREADS,
-                            (size_t)nmax * sizeof(To), cs>>>(
-        (const ChainTask<Ti, To> *)(base + o_tasks), nt, (int *)(base + o_next));
+    k_chain_batch<Ti, To><<<(unsigned)std::min(nt, 2 * 152 / CHAIN_CTAS) * CHAIN_CTAS, CHAIN_THREADS,
+                            (size_t)chain_smem(nmax) * sizeof(To), cs>>>(
+        (const ChainTask<Ti, To> *)(base + o_tasks), nt);
     ed_count_launches(1);
     if (nmats > 0) {
       k_cfrac_batch<<<dim3((nmats + 31) / 32, nt), 32, 0, cs>>>(
@@ -894,8 +922,7 @@ static ed_status chain_batch(ed_sector s, const Ti *psi, double e0, int nsteps, 
     t.psi = psi;
     t.nsteps = nsteps;
     off.push_back(bytes);
-    bytes += 3 * al256(nb->bdim * sizeof(To)) + al256(sizeof(LanczosState)) +
-             (shift ? ed_shift_diag_bytes(nb) : 0);
+    bytes += al256(sizeof(LanczosState)) + (shift ? ed_shift_diag_bytes(nb) : 0);
     nbs.push_back(nb);
     tasks.push_back(t);
     job_of.push_back(q);
@@ -903,7 +930,7 @@ static ed_status chain_batch(ed_sector s, const Ti *psi, double e0, int nsteps, 
   }
   const int nt = (int)tasks.size();
   if (nt == 0) return ED_OK;
-  // the chains' vectors and states, on this solve's stream
+  // the chains' states, on this solve's stream
   void *mem = nullptr;
   ED_TRY(ed_dmalloc(&mem, bytes + 256, cs, "batched chain workspace"));
   char *base = (char *)mem;
@@ -915,11 +942,7 @@ static ed_status chain_batch(ed_sector s, const Ti *psi, double e0, int nsteps, 
   m.stream = cs;
   for (int i = 0; i < nt; ++i) {
     char *p = base + off[i];
-    const size_t vb = al256(tasks[i].a.dst_dim * sizeof(To));
-    tasks[i].b0 = (To *)p;
-    tasks[i].b1 = (To *)(p + vb);
-    tasks[i].b2 = (To *)(p + 2 * vb);
-    tasks[i].st = (LanczosState *)(p + 3 * vb);
+    tasks[i].st = (LanczosState *)p;
     m.sts.push_back(tasks[i].st);
     m.sgn.push_back(sgn[i]);
     m.e0.push_back(shift ? 0.0 : e0);  // the continued fraction's e0 - sigma
@@ -928,9 +951,7 @@ static ed_status chain_batch(ed_sector s, const Ti *psi, double e0, int nsteps, 
   if constexpr (shift) {
     for (int i = 0; i < nt && rs == ED_OK; ++i)
       rs = ed_shift_diag32(nbs[i], e0,
-                           base + off[i] + 3 * al256(tasks[i].a.dst_dim * sizeof(To)) +
-                               al256(sizeof(LanczosState)),
-                           &tasks[i].tb, cs);
+                           base + off[i] + al256(sizeof(LanczosState)), &tasks[i].tb, cs);
   }
   if (rs != ED_OK) {
     ed_dfree(mem, cs);
