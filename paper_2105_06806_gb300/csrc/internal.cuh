@@ -337,6 +337,7 @@ struct HvTables {
   int nfib[2] = {0, 0};
   int64_t fib_first[2] = {0, 0}, fib_n[2] = {0, 0};
   int64_t row0 = 0, rows = 0;
+  bool dw_narrow = false;  // short tiles of the H_dw pass (k_hv_dw)
   T hop_up[ED_MAX_NS];
   // H_nd (spin exchange, pair hopping): move tables of this layout, or null
   const int32_t *nd_up = nullptr, *nd_dw = nullptr;

@@ -127,7 +127,13 @@ static int64_t small_grid_of(int64_t n) {
   return (nblk + k - 1) / k;
 }
 
+// H_dw pass of the two-pass product (k_hv_dw)
+constexpr int DW_THREADS = 256;
+constexpr int DW_ROWS = 32;    // rows of an item
+constexpr int DW_COLS = 512;   // columns of an item (a multiple of 4)
+
 static bool passa_is_wide(ed_sector s);
+static int64_t widest_block(ed_sector s);  // padded columns of the widest up block
 
 // fiber.cuh: launch of the orbital-factorised product (a = nullptr: prepare)
 namespace fiber {
@@ -220,6 +226,7 @@ HvTables<float> ed_hv_tables<float>(ed_sector s, int layout) {
   t.small_chunk = (int32_t)small_chunk_of(s->bdim);
   t.passa_wide = layout == 1 && passa_is_wide(s);
   t.fiber = il.fiber;
+  t.dw_narrow = il.fiber && widest_block(s) < 4 * DW_COLS;
   t.rows = s->sp[1].dim;
   for (int k = 0, b = 0; k < FIBER_SHAPES; b += il.nfib[k], ++k) {
     t.fib[k] = il.d_fib + b;
@@ -234,10 +241,6 @@ HvTables<float> ed_hv_tables<float>(ed_sector s, int layout) {
 }
 
 constexpr int HV_THREADS = 512;
-// H_dw pass of the two-pass product (k_hv_dw)
-constexpr int DW_THREADS = 256;
-constexpr int DW_ROWS = 32;    // rows of an item
-constexpr int DW_COLS = 512;   // columns of an item (a multiple of 4)
 constexpr size_t HV_SMEM_TWO = 88 * 1024;   // two CTAs per SM (with the static tables)
 constexpr size_t HV_SMEM_MAX = 190 * 1024;  // one CTA per SM (very wide blocks)
 constexpr int HV_MAXROWS = 64;              // rows of an item (G * RT <= 16 * 4)
@@ -434,12 +437,13 @@ static bool two_pass_wanted(ed_sector s, int elem) {
 }
 
 // the H_up pass shape of this sector (see rt_passa)
-static bool passa_is_wide(ed_sector s) {
+static int64_t widest_block(ed_sector s) {
   int64_t w = 0;
   for (size_t k = 0; k + 1 < s->up_off_pad.size(); ++k)
     w = std::max<int64_t>(w, s->up_off_pad[k + 1] - s->up_off_pad[k]);
-  return w > (int64_t)EDGB_PASSA_WIDE;
+  return w;
 }
+static bool passa_is_wide(ed_sector s) { return widest_block(s) > (int64_t)EDGB_PASSA_WIDE; }
 
 // CTA shape of the orbital-factorised product for an up block of padded width
 // w: the smallest one with room for a row; -1: none
@@ -1126,9 +1130,13 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
 // the first pass's value and adds the H_dw terms in the same order as k_hv,
 // so the product equals the one-pass product bit for bit.
 
-template <typename T, int MODE>
+//
+// A thread takes RT rows x 4 columns, NB neighbour rows in flight.  Blocks
+// narrower than an item leave most threads of a tall tile without work: there
+// one row and 4 neighbours (Norb=3 Ns=15 168 -> 151 us, Norb=5 343 -> 246 us),
+// else Tile::RT rows and 2 (Norb=2 Ns=16 478 against 524 us).
+template <typename T, int MODE, int RT, int NB>
 __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
-  constexpr int RT = Tile<T>::RT;
   __shared__ double red[MODE == HV_LANCZOS ? DW_THREADS : 1];
   __shared__ int32_t s_dcol[DW_ROWS * ED_MAX_NS];
   __shared__ T s_dval[DW_ROWS * ED_MAX_NS];
@@ -1194,12 +1202,12 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
       const int32_t *dc = s_dcol + (lr0 + i) * ED_MAX_NS;
       const T *dv = s_dval + (lr0 + i) * ED_MAX_NS;
       int t = 0;
-      for (; t + 2 <= n; t += 2) {
-        T y[2][4];
-        load4(g + (int64_t)dc[t] * stride + col0, y[0]);
-        load4(g + (int64_t)dc[t + 1] * stride + col0, y[1]);
+      for (; t + NB <= n; t += NB) {
+        T y[NB][4];
 #pragma unroll
-        for (int q2 = 0; q2 < 2; ++q2) {
+        for (int q2 = 0; q2 < NB; ++q2) load4(g + (int64_t)dc[t + q2] * stride + col0, y[q2]);
+#pragma unroll
+        for (int q2 = 0; q2 < NB; ++q2) {
           const T h = dv[t + q2];
 #pragma unroll
           for (int u = 0; u < 4; ++u) acc[i][u] = fma_t<T>(h, y[q2][u], acc[i][u]);
@@ -1391,6 +1399,15 @@ template ed_status ed_hv_prepare<float>();
 template ed_status ed_hv_prepare<double>();
 
 template <typename T, int MODE>
+static void launch_dw(const HvLaunch<T> &a, unsigned ns, cudaStream_t st) {
+  const dim3 grid((unsigned)a.tb.nditems, ns);
+  if (a.tb.dw_narrow)
+    k_hv_dw<T, MODE, 1, 4><<<grid, DW_THREADS, 0, st>>>(a);
+  else
+    k_hv_dw<T, MODE, Tile<T>::RT, 2><<<grid, DW_THREADS, 0, st>>>(a);
+}
+
+template <typename T, int MODE>
 static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st) {
   if (a.tb.small_cols) {
     if (a.tb.small_chunk > 1)
@@ -1401,7 +1418,7 @@ static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st)
     if constexpr (sizeof(T) == 4) {
       ED_TRY(launch_fiber(a.tb.fiber, &a, MODE, ns, st));
     }
-    k_hv_dw<T, MODE><<<dim3((unsigned)a.tb.nditems, ns), DW_THREADS, 0, st>>>(a);
+    launch_dw<T, MODE>(a, ns, st);
   } else if (a.tb.ditems) {
     if (a.tb.passa_wide)
       k_hv<T, MODE, true, true, rt_passa<T, true>(), passa_threads<true>()>
@@ -1410,7 +1427,7 @@ static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st)
       k_hv<T, MODE, true, true, rt_passa<T, false>(), passa_threads<false>()>
           <<<dim3((unsigned)a.tb.nitems, ns), passa_threads<false>(), a.tb.smem, st>>>(a);
     ED_LAUNCHED(1);
-    k_hv_dw<T, MODE><<<dim3((unsigned)a.tb.nditems, ns), DW_THREADS, 0, st>>>(a);
+    launch_dw<T, MODE>(a, ns, st);
   } else if (a.tb.ell_col) {
     k_hv<T, MODE, true><<<dim3((unsigned)a.tb.nitems, ns), HV_THREADS, a.tb.smem, st>>>(a);
   } else {
