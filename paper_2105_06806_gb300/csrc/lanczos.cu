@@ -798,6 +798,22 @@ struct StreamJoin {
   }
 };
 
+// Zeros at the padding columns of a block-major vector (at most 3 per up block,
+// of which no supported model has more than 381).
+constexpr int ED_MAX_PAD_COLS = 1200;
+template <typename T>
+__global__ void k_clear_padding(T *v, int64_t rows, int64_t stride, const int32_t *padinv) {
+  __shared__ int32_t pad[ED_MAX_PAD_COLS];
+  __shared__ int npad;
+  if (threadIdx.x == 0) npad = 0;
+  __syncthreads();
+  for (int64_t c = threadIdx.x; c < stride; c += blockDim.x)
+    if (padinv[c] < 0) pad[atomicAdd(&npad, 1)] = (int32_t)c;
+  __syncthreads();
+  for (int64_t r = blockIdx.x; r < rows; r += gridDim.x)
+    for (int k = threadIdx.x; k < npad; k += blockDim.x) v[r * stride + pad[k]] = T(0);
+}
+
 // Krylov basis kept on the device during the first pass, so that the ground
 // state needs no second pass (the paper's second pass trades a second run of
 // the recurrence for memory; this part has the memory).  Vectors are
@@ -818,6 +834,7 @@ struct BasisStore {
   bool full = false;             // budget reached: nothing more is stored
   int filled = 0;                // table entries uploaded
   size_t vbytes = 0, budget = 0, used = 0;
+  ed_sector s = nullptr;
   cudaStream_t st = nullptr;
   ~BasisStore() {
     for (void *p : owned) ed_dfree(p, st);
@@ -840,7 +857,12 @@ struct BasisStore {
         } else {
           owned.push_back(q);
           used += vbytes;
-          ED_TRY_CUDA(cudaMemsetAsync(q, 0, vbytes, cs));  // padding entries stay zero
+          // padding entries stay zero; the others are written before they are read
+          if (s->bstride > s->sp[0].dim) {
+            k_clear_padding<T><<<(unsigned)std::min<int64_t>(s->sp[1].dim, 152 * 8), 128, 0, cs>>>(
+                (T *)q, s->sp[1].dim, s->bstride, s->padinv);
+            ED_LAUNCHED(1);
+          }
           p = (T *)q;
           cap = j + 1;
         }
@@ -1037,6 +1059,7 @@ static ed_status lanczos_solve(ed_sector s, int maxit, double tol, uint64_t seed
     coef = (T *)p;
     bs.table.assign(maxit + 2, nullptr);
     bs.v0 = bufs[0];
+    bs.s = s;
     bs.rot[0] = psi;
     bs.rot[1] = bufs[1];
     bs.rot[2] = bufs[2];

@@ -117,13 +117,20 @@ constexpr int HVS_THREADS = 256;
 #ifndef EDGB_SMALL_PARTS
 #define EDGB_SMALL_PARTS (1 << 16)
 #endif
-static int64_t small_chunk_of(int64_t n) {
+// The Lanczos mode caps them lower: its partials are summed by one CTA, on one
+// SM's FP64 lanes (46,000 partials: 20 us), and every CTA's own sum costs FP64
+// issue.
+#ifndef EDGB_SMALL_LANCZOS_PARTS
+#define EDGB_SMALL_LANCZOS_PARTS (1 << 13)
+#endif
+static int64_t small_chunk_of(int64_t n, bool lanczos) {
   const int64_t nblk = (n + HVS_THREADS - 1) / HVS_THREADS;
-  return std::max<int64_t>(1, (nblk + EDGB_SMALL_PARTS - 1) / EDGB_SMALL_PARTS);
+  const int64_t parts = lanczos ? EDGB_SMALL_LANCZOS_PARTS : EDGB_SMALL_PARTS;
+  return std::max<int64_t>(1, (nblk + parts - 1) / parts);
 }
-static int64_t small_grid_of(int64_t n) {
+static int64_t small_grid_of(int64_t n, bool lanczos) {
   const int64_t nblk = (n + HVS_THREADS - 1) / HVS_THREADS;
-  const int64_t k = small_chunk_of(n);
+  const int64_t k = small_chunk_of(n, lanczos);
   return (nblk + k - 1) / k;
 }
 
@@ -200,8 +207,10 @@ HvTables<double> ed_hv_tables<double>(ed_sector s, int layout) {
   t.ell_col = layout == 0 ? nullptr : s->ell_col;
   t.ell_val = layout == 0 ? nullptr : s->ell_v64;
   t.small_cols = (layout == 1 && s->hv_kernel[1] == 1) ? s->small_cols : nullptr;
-  t.small_grid = t.small_cols ? small_grid_of(s->bdim) : 0;
-  t.small_chunk = (int32_t)small_chunk_of(s->bdim);
+  for (int k = 0; k < 2; ++k) {
+    t.small_grid[k] = t.small_cols ? small_grid_of(s->bdim, k == 1) : 0;
+    t.small_chunk[k] = (int32_t)small_chunk_of(s->bdim, k == 1);
+  }
   t.passa_wide = layout == 1 && passa_is_wide(s);
   set_nd<double>(t, s, layout);
   return t;
@@ -222,8 +231,10 @@ HvTables<float> ed_hv_tables<float>(ed_sector s, int layout) {
   t.ell_col = layout == 0 ? nullptr : s->ell_col;
   t.ell_val = layout == 0 ? nullptr : s->ell_v32;
   t.small_cols = (layout == 1 && s->hv_kernel[0] == 1) ? s->small_cols : nullptr;
-  t.small_grid = t.small_cols ? small_grid_of(s->bdim) : 0;
-  t.small_chunk = (int32_t)small_chunk_of(s->bdim);
+  for (int k = 0; k < 2; ++k) {
+    t.small_grid[k] = t.small_cols ? small_grid_of(s->bdim, k == 1) : 0;
+    t.small_chunk[k] = (int32_t)small_chunk_of(s->bdim, k == 1);
+  }
   t.passa_wide = layout == 1 && passa_is_wide(s);
   t.fiber = il.fiber;
   t.dw_narrow = il.fiber && widest_block(s) < 4 * DW_COLS;
@@ -1296,7 +1307,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
   const int64_t n = tb.ddw * stride;
   // one element per thread unless CHUNKED (separate instances: the chunk loop
   // costs registers, and the small sectors run at full occupancy without it)
-  const int K = CHUNKED ? tb.small_chunk : 1;
+  const int K = CHUNKED ? tb.small_chunk[MODE == HV_LANCZOS] : 1;
   for (int k = 0; k < K; ++k) {
     const int64_t gi = ((int64_t)blockIdx.x * K + k) * HVS_THREADS + threadIdx.x;
     if (gi >= n) break;
@@ -1346,7 +1357,7 @@ int64_t ed_hv_num_parts(ed_sector s, int layout, int elem_size) {
   if (ed_build_items(s, layout, elem_size) != ED_OK) return 0;
   // the H_nd kernel's partials follow the product's
   const int64_t nd = s->nd[layout].up ? ed_nd_grid(s->sp[1].dim, s->nd[layout].ncols) : 0;
-  if (layout == 1 && s->hv_kernel[elem_size == 8 ? 1 : 0] == 1) return small_grid_of(s->bdim) + nd;
+  if (layout == 1 && s->hv_kernel[elem_size == 8 ? 1 : 0] == 1) return small_grid_of(s->bdim, true) + nd;
   const ItemList &il = s->items[layout][elem_size == 8 ? 1 : 0];
   return (il.d_ditems ? il.nditems : il.nitems) + nd;
 }
@@ -1410,10 +1421,11 @@ static void launch_dw(const HvLaunch<T> &a, unsigned ns, cudaStream_t st) {
 template <typename T, int MODE>
 static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st) {
   if (a.tb.small_cols) {
-    if (a.tb.small_chunk > 1)
-      k_hv_small<T, MODE, true><<<dim3((unsigned)a.tb.small_grid, ns), HVS_THREADS, 0, st>>>(a);
+    constexpr int L = MODE == HV_LANCZOS;
+    if (a.tb.small_chunk[L] > 1)
+      k_hv_small<T, MODE, true><<<dim3((unsigned)a.tb.small_grid[L], ns), HVS_THREADS, 0, st>>>(a);
     else
-      k_hv_small<T, MODE, false><<<dim3((unsigned)a.tb.small_grid, ns), HVS_THREADS, 0, st>>>(a);
+      k_hv_small<T, MODE, false><<<dim3((unsigned)a.tb.small_grid[L], ns), HVS_THREADS, 0, st>>>(a);
   } else if (a.tb.fiber) {
     if constexpr (sizeof(T) == 4) {
       ED_TRY(launch_fiber(a.tb.fiber, &a, MODE, ns, st));
@@ -1447,7 +1459,7 @@ ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v,
   HvLaunch<T> a;
   a.tb = tb;
   // CTAs of the (last) product kernel = its partial sums in the Lanczos mode
-  const int64_t np = tb.small_cols ? tb.small_grid
+  const int64_t np = tb.small_cols ? tb.small_grid[mode == HV_LANCZOS]
                                    : (tb.ditems ? tb.nditems : tb.nitems);
   if (nparts) *nparts = np;
   if ((tb.fiber ? tb.rows : tb.nitems) == 0 || tb.dup == 0) return ED_OK;
