@@ -223,10 +223,23 @@ def kernel_launches() -> int:
     return int(lib().ed_kernel_launches())
 
 
+_current_stream = None
+
+
+def _resolve_current_stream():
+    """Address of the current stream of the current device, without building a
+    Stream object (half of the host time of a small product's call)."""
+    global _current_stream
+    import torch
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+    _current_stream = ((lambda: raw(device())) if raw is not None
+                       else (lambda: torch.cuda.current_stream().cuda_stream))
+    return _current_stream()
+
+
 def _stream_ptr(stream=None):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return (_current_stream or _resolve_current_stream)()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -357,22 +370,25 @@ def _psi_ptr(psi, precision):
     return C.c_void_p(psi.data_ptr())
 
 
+def _matvec(f, name, sector, v, w, precision, stream):
+    # a small product is bound by this host code: integers go to the C call as
+    # they are
+    n = v.numel()
+    if n != w.numel():
+        raise ValueError("v and w differ in length")
+    st = f(sector.h, _prec(precision), v.data_ptr(), w.data_ptr(), n, _stream_ptr(stream))
+    if st != ED_OK:
+        raise EDError(st, name)
+
+
 def matvec(sector: Sector, v, w, precision="fp64", stream=None):
     """w = H v for device tensors (float64 for fp64, float32 otherwise)."""
-    if v.numel() != w.numel():
-        raise ValueError("v and w differ in length")
-    _check(lib().ed_matvec(sector.h, _prec(precision), C.c_void_p(v.data_ptr()),
-                           C.c_void_p(w.data_ptr()), int(v.numel()),
-                           C.c_void_p(_stream_ptr(stream))), "ed_matvec")
+    _matvec(lib().ed_matvec, "ed_matvec", sector, v, w, precision, stream)
 
 
 def matvec_blocked(sector: Sector, v, w, precision="fp64", stream=None):
     """w = H v with both vectors in block-major order."""
-    if v.numel() != w.numel():
-        raise ValueError("v and w differ in length")
-    _check(lib().ed_matvec_blocked(sector.h, _prec(precision), C.c_void_p(v.data_ptr()),
-                                   C.c_void_p(w.data_ptr()), int(v.numel()),
-                                   C.c_void_p(_stream_ptr(stream))), "ed_matvec_blocked")
+    _matvec(lib().ed_matvec_blocked, "ed_matvec_blocked", sector, v, w, precision, stream)
 
 
 def permute(sector: Sector, x, out, to_blocked=True, precision="fp64", stream=None):
