@@ -436,8 +436,13 @@ struct LanczosState {
   double cvv;         // <v_j, v_{j-1}>, from the update of the previous step
 };
 
-// Modes of the fused product kernel.
-enum { HV_PLAIN = 0, HV_LANCZOS = 1, HV_SECOND = 2 };
+// Modes of the fused product kernel.  HV_SLICED (kernels only): HV_PLAIN on
+// several slices, grid row y on slice y; its own instances, because the two
+// shifted pointers cost HV_PLAIN registers at its cap (2-4% of large products).
+enum { HV_PLAIN = 0, HV_LANCZOS = 1, HV_SECOND = 2, HV_SLICED = 4 };
+__host__ __device__ constexpr bool ed_hv_plain(int mode) {
+  return mode == HV_PLAIN || mode == HV_SLICED;
+}
 
 template <typename T>
 ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v, T *w,

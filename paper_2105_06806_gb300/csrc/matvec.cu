@@ -922,9 +922,9 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
   __shared__ EpState ep_s;
   const T *g;
   T *out_plain = nullptr;
-  if (MODE == HV_PLAIN) {
-    g = a.v + blockIdx.y * a.slice;
-    out_plain = a.w + blockIdx.y * a.slice;
+  if (ed_hv_plain(MODE)) {
+    g = MODE == HV_SLICED ? a.v + blockIdx.y * a.slice : a.v;
+    out_plain = MODE == HV_SLICED ? a.w + blockIdx.y * a.slice : a.w;
   } else {
     const LanczosState *st = a.st;
     if (MODE == HV_LANCZOS && st->done) return;
@@ -1025,8 +1025,8 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
       // sector-order layout is not aligned: element accesses there)
       const bool vec = BLK && full;
       const volatile EpState &ep = ep_s;
-      T *const out = MODE == HV_PLAIN ? out_plain : ep.out;
-      if (MODE == HV_PLAIN || PASSA) {
+      T *const out = ed_hv_plain(MODE) ? out_plain : ep.out;
+      if (ed_hv_plain(MODE) || PASSA) {
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
           if (i >= nrt) continue;
@@ -1158,9 +1158,9 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
   const T *g;
   const T *prev = nullptr;
   T *out;
-  if (MODE == HV_PLAIN) {
-    g = a.v + blockIdx.y * a.slice;
-    out = a.w + blockIdx.y * a.slice;
+  if (ed_hv_plain(MODE)) {
+    g = MODE == HV_SLICED ? a.v + blockIdx.y * a.slice : a.v;
+    out = MODE == HV_SLICED ? a.w + blockIdx.y * a.slice : a.w;
   } else {
     const LanczosState *st = a.st;
     if (MODE == HV_LANCZOS && st->done) return;
@@ -1240,7 +1240,7 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
       for (int u = 0; u < 4; ++u) {
         if (cb + u >= it.nc) continue;  // padding is not written
         const int64_t gi = rowbase + u;
-        if (MODE == HV_PLAIN) {
+        if (ed_hv_plain(MODE)) {
           out[gi] = acc[i][u];
         } else {
           const T x = g[gi];
@@ -1278,9 +1278,9 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
   const T *g;
   const T *prev = nullptr;
   T *out;
-  if (MODE == HV_PLAIN) {
-    g = a.v + blockIdx.y * a.slice;
-    out = a.w + blockIdx.y * a.slice;
+  if (ed_hv_plain(MODE)) {
+    g = MODE == HV_SLICED ? a.v + blockIdx.y * a.slice : a.v;
+    out = MODE == HV_SLICED ? a.w + blockIdx.y * a.slice : a.w;
   } else {
     const LanczosState *st = a.st;
     if (MODE == HV_LANCZOS && st->done) return;
@@ -1331,7 +1331,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
       const int32_t d0 = __ldg(tb.rp_dw + r), d1 = __ldg(tb.rp_dw + r + 1);
       for (int32_t k = d0; k < d1; ++k)
         acc = fma_t<T>(__ldg(tb.val_dw + k), g[(int64_t)__ldg(tb.col_dw + k) * stride + pc], acc);
-      if (MODE == HV_PLAIN) {
+      if (ed_hv_plain(MODE)) {
         out[gi] = acc;
       } else {
         T w1 = mul_t<T>(acc, s_cur);
@@ -1369,6 +1369,8 @@ static ed_status prepare_passa() {
   constexpr int RT = rt_passa<T, WIDE>(), NT = passa_threads<WIDE>();
   ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_PLAIN, true, true, RT, NT>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
+  ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_SLICED, true, true, RT, NT>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
   ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_LANCZOS, true, true, RT, NT>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
   ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_SECOND, true, true, RT, NT>,
@@ -1379,6 +1381,8 @@ static ed_status prepare_passa() {
 template <typename T, bool BLK>
 static ed_status prepare_layout() {
   ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_PLAIN, BLK>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
+  ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_SLICED, BLK>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
   ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_LANCZOS, BLK>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
@@ -1428,7 +1432,7 @@ static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st)
       k_hv_small<T, MODE, false><<<dim3((unsigned)a.tb.small_grid[L], ns), HVS_THREADS, 0, st>>>(a);
   } else if (a.tb.fiber) {
     if constexpr (sizeof(T) == 4) {
-      ED_TRY(launch_fiber(a.tb.fiber, &a, MODE, ns, st));
+      ED_TRY(launch_fiber(a.tb.fiber, &a, ed_hv_plain(MODE) ? HV_PLAIN : MODE, ns, st));
     }
     launch_dw<T, MODE>(a, ns, st);
   } else if (a.tb.ditems) {
@@ -1474,7 +1478,9 @@ ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v,
   a.st = state;
   a.part = part;
   a.slice = slice;
-  if (mode == HV_PLAIN) ED_TRY((launch_mode<T, HV_PLAIN>(a, (unsigned)nslices, st)));
+  if (mode == HV_PLAIN && nslices > 1)
+    ED_TRY((launch_mode<T, HV_SLICED>(a, (unsigned)nslices, st)));
+  else if (mode == HV_PLAIN) ED_TRY((launch_mode<T, HV_PLAIN>(a, 1, st)));
   else if (mode == HV_LANCZOS) ED_TRY((launch_mode<T, HV_LANCZOS>(a, 1, st)));
   else ED_TRY((launch_mode<T, HV_SECOND>(a, 1, st)));
   if (!tb.nd_up) return ED_OK;

@@ -62,7 +62,7 @@ struct HvLaunch {
   T *psi;
   LanczosState *st;
   double *part;
-  int64_t slice = 0;  // HV_PLAIN: grid row y works on v + y * slice, w + y * slice
+  int64_t slice = 0;  // HV_SLICED: grid row y works on v + y * slice, w + y * slice
 };
 
 // Sum over a CTA of NT threads (fixed order), in thread 0 of the first warp:
