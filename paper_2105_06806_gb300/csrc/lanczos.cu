@@ -616,31 +616,46 @@ __global__ void k_scale_copy(const Ti *x, To *y, int64_t n, const double *part, 
 // padded block-major order ([D_dw][bstride]):
 //   blocked[r'][pc] = sector[pidx_dw[r']][pidx_up[padinv[pc]]]  (0 at padding)
 //   sector[r][c]    = blocked[inv_dw[r]][colpos[inv_up[c]]]
-// One grid row per output row; the gathers stay inside one input row.
+// Bound: HBM (each element read and written once, the gathers stay inside one
+// input row).  A thread takes one column of PERM_ROWS rows, so that its source
+// column is looked up once and the rows' loads are in flight together (one
+// element per thread waited for the tables and then for the element): Norb=2 Ns=16 FP32 0.84 -> 0.41 ms into and 1.07 -> 0.55
+// ms out of block-major order.
+constexpr int PERM_ROWS = 8, PERM_THREADS = 256;
 template <typename Ti, typename To>
-__global__ void k_to_blocked(const Ti *in, To *out, const int32_t *pidx_dw,
-                             const int32_t *pidx_up, const int32_t *padinv, int64_t dup,
-                             int64_t stride, int64_t ddw) {
-  for (int64_t r = blockIdx.y; r < ddw; r += gridDim.y) {
-    const Ti *src = in + (int64_t)pidx_dw[r] * dup;
-    To *dst = out + r * stride;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < stride;
-         c += (int64_t)gridDim.x * blockDim.x) {
-      const int32_t cb = padinv[c];
-      dst[c] = cb < 0 ? To(0) : (To)src[pidx_up[cb]];
-    }
+__global__ void __launch_bounds__(PERM_THREADS) k_to_blocked(
+    const Ti *in, To *out, const int32_t *pidx_dw, const int32_t *pidx_up, const int32_t *padinv,
+    int64_t dup, int64_t stride, int64_t ddw) {
+  const int64_t c = blockIdx.x * (int64_t)PERM_THREADS + threadIdx.x;
+  if (c >= stride) return;
+  const int32_t cb = padinv[c];
+  const int64_t src = cb < 0 ? 0 : pidx_up[cb];
+  for (int64_t r0 = (int64_t)blockIdx.y * PERM_ROWS; r0 < ddw; r0 += (int64_t)gridDim.y * PERM_ROWS) {
+    Ti x[PERM_ROWS];
+#pragma unroll
+    for (int k = 0; k < PERM_ROWS; ++k)
+      x[k] = r0 + k < ddw ? __ldg(in + __ldg(pidx_dw + r0 + k) * dup + src) : Ti(0);
+#pragma unroll
+    for (int k = 0; k < PERM_ROWS; ++k)
+      if (r0 + k < ddw) out[(r0 + k) * stride + c] = cb < 0 ? To(0) : (To)x[k];
   }
 }
 
 template <typename Ti, typename To>
-__global__ void k_from_blocked(const Ti *in, To *out, const int32_t *inv_dw, const int32_t *inv_up,
-                               const int32_t *colpos, int64_t dup, int64_t stride, int64_t ddw) {
-  for (int64_t r = blockIdx.y; r < ddw; r += gridDim.y) {
-    const Ti *src = in + (int64_t)inv_dw[r] * stride;
-    To *dst = out + r * dup;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < dup;
-         c += (int64_t)gridDim.x * blockDim.x)
-      dst[c] = (To)src[colpos[inv_up[c]]];
+__global__ void __launch_bounds__(PERM_THREADS) k_from_blocked(
+    const Ti *in, To *out, const int32_t *inv_dw, const int32_t *inv_up, const int32_t *colpos,
+    int64_t dup, int64_t stride, int64_t ddw) {
+  const int64_t c = blockIdx.x * (int64_t)PERM_THREADS + threadIdx.x;
+  if (c >= dup) return;
+  const int64_t src = colpos[inv_up[c]];
+  for (int64_t r0 = (int64_t)blockIdx.y * PERM_ROWS; r0 < ddw; r0 += (int64_t)gridDim.y * PERM_ROWS) {
+    Ti x[PERM_ROWS];
+#pragma unroll
+    for (int k = 0; k < PERM_ROWS; ++k)
+      x[k] = r0 + k < ddw ? __ldg(in + __ldg(inv_dw + r0 + k) * stride + src) : Ti(0);
+#pragma unroll
+    for (int k = 0; k < PERM_ROWS; ++k)
+      if (r0 + k < ddw) out[(r0 + k) * dup + c] = (To)x[k];
   }
 }
 
@@ -649,14 +664,15 @@ static ed_status permute_layout(ed_sector s, const Ti *in, To *out, bool to_bloc
                                 cudaStream_t cs) {
   const int64_t dup = s->sp[0].dim, ddw = s->sp[1].dim, stride = s->bstride;
   const int64_t cols = to_blocked ? stride : dup;
-  dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>((cols + 255) / 256, 64)),
-            (unsigned)std::max<int64_t>(1, std::min<int64_t>(ddw, 65535)));
+  dim3 grid((unsigned)std::max<int64_t>(1, (cols + PERM_THREADS - 1) / PERM_THREADS),
+            (unsigned)std::max<int64_t>(
+                1, std::min<int64_t>((ddw + PERM_ROWS - 1) / PERM_ROWS, 65535)));
   if (to_blocked)
-    k_to_blocked<Ti, To><<<grid, 256, 0, cs>>>(in, out, s->bi[1].pidx, s->bi[0].pidx, s->padinv,
-                                               dup, stride, ddw);
+    k_to_blocked<Ti, To><<<grid, PERM_THREADS, 0, cs>>>(in, out, s->bi[1].pidx, s->bi[0].pidx,
+                                                        s->padinv, dup, stride, ddw);
   else
-    k_from_blocked<Ti, To><<<grid, 256, 0, cs>>>(in, out, s->bi[1].inv, s->bi[0].inv, s->colpos,
-                                                 dup, stride, ddw);
+    k_from_blocked<Ti, To><<<grid, PERM_THREADS, 0, cs>>>(in, out, s->bi[1].inv, s->bi[0].inv,
+                                                          s->colpos, dup, stride, ddw);
   ED_LAUNCHED(1);
   return ED_OK;
 }
