@@ -619,8 +619,8 @@ __global__ void k_scale_copy(const Ti *x, To *y, int64_t n, const double *part, 
 // Bound: HBM (each element read and written once, the gathers stay inside one
 // input row).  A thread takes one column of PERM_ROWS rows, so that its source
 // column is looked up once and the rows' loads are in flight together (one
-// element per thread waited for the tables and then for the element): Norb=2 Ns=16 FP32 0.84 -> 0.41 ms into and 1.07 -> 0.55
-// ms out of block-major order.
+// element per thread waited for the tables and then for the element): Norb=2
+// Ns=16 FP32 0.84 -> 0.41 ms into and 1.07 -> 0.55 ms out of block-major order.
 constexpr int PERM_ROWS = 8, PERM_THREADS = 256;
 template <typename Ti, typename To>
 __global__ void __launch_bounds__(PERM_THREADS) k_to_blocked(
@@ -914,9 +914,14 @@ static ed_status run_steps(ed_sector s, const HvTables<T> &tb, T *const *bufs, L
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   ED_TRY(ed_hv_prepare<T>());
-  // product kernels per step: two for the two-pass product, else one; plus
-  // the H_nd kernel with spin exchange or pair hopping
-  const int64_t hv_per_step = ((tb.ditems && !tb.small_cols) ? 2 : 1) + (tb.nd_up ? 1 : 0);
+  // product kernels per step: H_up (a launch per CTA shape of the
+  // orbital-factorised product) and H_dw passes, else one; plus the H_nd kernel
+  // with spin exchange or pair hopping
+  const int64_t hv_per_step =
+      (tb.small_cols || !tb.ditems
+           ? 1
+           : (tb.fiber ? (tb.fib_n[0] > 0) + (tb.fib_n[1] > 0) : 1) + 1) +
+      (tb.nd_up ? 1 : 0);
   ED_TRY_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
   ed_status rs = ED_OK;
   for (int it = 0; it < chunk && rs == ED_OK; ++it) {

@@ -556,6 +556,17 @@ __global__ void k_tune_fill(T *v, int64_t n, int64_t stride, const int32_t *padi
   }
 }
 
+// True when this sector's kernel is known to be the tiled family without timing
+// anything.
+static bool tuned_tiled(ed_sector s, int elem) {
+  const int8_t k = s->hv_kernel[elem == 8 ? 1 : 0];
+  if (k >= 0) return k == 0;
+  if (s->bdim <= (int64_t)EDGB_TUNE_MIN) return false;
+  std::lock_guard<std::mutex> lk(g_tune_mu);
+  const auto it = g_tune.find(TuneKey{s->mp.norb, s->mp.nbath, elem});
+  return it != g_tune.end() && it->second == 0;
+}
+
 template <typename T>
 static ed_status time_hv_kernels(ed_sector s, int e, cudaStream_t cs, double ms[2]) {
   const int64_t n = s->bdim;
@@ -665,8 +676,12 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
     op_up = ob_up;
     ob_dw = {0, s->sp[1].dim};
   } else {
-    ED_TRY(ed_build_ell(s, cs));
-    ED_TRY(build_small_cols(s, cs));
+    // the orbital-factorised product reads no table of H_up: where the shape is
+    // known to take it, the ELL table waits until something else needs it
+    if (!(elem == 4 && fiber_group(s) && tuned_tiled(s, elem))) {
+      ED_TRY(ed_build_ell(s, cs));
+      ED_TRY(build_small_cols(s, cs));
+    }
     ob_up = s->bi[0].offset;
     op_up = s->up_off_pad;
     ob_dw = s->bi[1].offset;
@@ -1499,6 +1514,46 @@ template ed_status ed_launch_hv<double>(ed_sector, const HvTables<double> &, int
                                         double *, int64_t *, cudaStream_t, double *const *, int,
                                         int64_t);
 
+// Sector-order FP32 product through block-major order: both permutations and
+// the orbital-factorised product in a scratch pair of vectors.  From
+// EDGB_PERMUTE_MIN elements this beats the sector-order kernel, whose H_up
+// hops gather across whole CSR rows (Norb=2 Ns=14 (5,6): 88
+// against 97 us, Norb=2 Ns=16 1.93 against 2.72 ms).
+// *done = false: not taken (the kernel choice, no memory for the scratch, or a
+// stream under capture, where the scratch would become part of the graph).
+#ifndef EDGB_PERMUTE_MIN
+#define EDGB_PERMUTE_MIN (1 << 20)
+#endif
+static ed_status matvec_permuted(ed_sector s, const float *v, float *w, cudaStream_t st,
+                                 bool *done) {
+  *done = false;
+  if (s->mp.norb < 2 || s->dim < (int64_t)EDGB_PERMUTE_MIN) return ED_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return ED_OK;
+  }
+  // both layouts' work lists, so that a later call under capture builds nothing
+  ED_TRY(ed_build_items(s, 0, 4));
+  ED_TRY(ed_build_items(s, 1, 4));
+  const HvTables<float> tb = ed_hv_tables<float>(s, 1);
+  if (!tb.fiber || tb.small_cols) return ED_OK;
+  void *mem = nullptr;
+  if (ed_dmalloc(&mem, 2 * s->bdim * sizeof(float), st, "permuted product") != ED_OK) {
+    cudaGetLastError();
+    ed_set_error_msg("");
+    return ED_OK;
+  }
+  float *bv = (float *)mem, *bw = bv + s->bdim;
+  ed_status rs = ed_permute_vec(s, ED_FP32, true, v, bv, st);
+  if (rs == ED_OK)
+    rs = ed_launch_hv<float>(s, tb, HV_PLAIN, bv, bw, nullptr, nullptr, nullptr, nullptr, nullptr, st);
+  if (rs == ED_OK) rs = ed_permute_vec(s, ED_FP32, false, bw, w, st);
+  ed_dfree(mem, st);
+  *done = rs == ED_OK;
+  return rs;
+}
+
 static ed_status matvec_layout(ed_sector s, ed_precision prec, const void *d_v, void *d_w,
                                int64_t n, void *stream, int layout) {
   if (!s || !d_v || !d_w || d_v == d_w) return ED_ERR_ARG;
@@ -1525,6 +1580,9 @@ static ed_status matvec_layout(ed_sector s, ed_precision prec, const void *d_v, 
                                 nullptr, nullptr, st);
   }
   if (prec == ED_FP32 || prec == ED_FP32_POLISH) {
+    bool done = false;
+    if (layout == 0) ED_TRY(matvec_permuted(s, (const float *)d_v, (float *)d_w, st, &done));
+    if (done) return ED_OK;
     ED_TRY(ed_build_items(s, layout, 4));
     return ed_launch_hv<float>(s, ed_hv_tables<float>(s, layout), HV_PLAIN, (const float *)d_v,
                                (float *)d_w, nullptr, nullptr, nullptr, nullptr, nullptr, st);
@@ -1575,6 +1633,11 @@ extern "C" ed_status ed_sector_set_kernel(ed_sector s, ed_precision prec, int32_
   int32_t cur = 0;
   ED_TRY(kernel_of(s, prec, &e, &cur));
   if (kernel == ED_KERNEL_ELEMENTWISE) {
+    ed_status ps = ED_OK;
+    cudaStream_t cs = ed_private_stream(&ps);
+    if (ps != ED_OK) return ps;
+    ED_TRY(ed_build_ell(s, cs));
+    ED_TRY(build_small_cols(s, cs));
     if (!s->small_cols) {
       ed_set_error_msg("this sector's blocks do not fit the element-parallel column table");
       return ED_ERR_UNSUPPORTED;
