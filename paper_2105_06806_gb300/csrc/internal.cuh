@@ -327,7 +327,8 @@ struct HvTables {
   int64_t nditems;
   const int4 *small_cols;  // non-null: element-parallel product (small sectors)
   int64_t small_grid[2];   // its CTAs, [1] in the Lanczos mode (= block partials)
-  int32_t small_chunk[2];  // its elements per thread
+  int32_t small_chunk[2];  // its elements (small_rows: columns of 4 rows) per thread
+  bool small_rows;         // 4 rows per thread (k_hv_rows)
   bool passa_wide;         // two-pass product: the wide shape of the H_up pass
   // orbital-factorised product (fiber.cuh): group size, 0 where not used; per CTA
   // shape the up blocks, the number of the first item and the items; the rows;
