@@ -380,7 +380,7 @@ def run_ours(args):
                      "unit": "GB/s", "frac": round(achieved / hbm, 4),
                      "traffic": _profiled_traffic(args.workload),
                      "kernel": "FP32 block-major product w = H v (ed_matvec_blocked"
-                               + (": H_up pass + H_dw pass)" if D > 1e9 else ", k_hv)"),
+                               + (": H_up pass + H_dw pass)" if m.norb > 1 else ", k_hv)"),
                      "peak_source": src, "products_ms": mv,
                      "kernel_ms": round(mv_ms, 4), "algorithmic_bytes": int(alg)},
         "e2e": e2e, "gpu_launches": int(launches), "clocks": clk,

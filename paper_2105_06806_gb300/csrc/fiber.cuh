@@ -25,7 +25,7 @@
 // Bound: shared-memory wavefronts (about 14 words per element: staging, two or
 // three accesses per axis, output) and the barriers between the axes; without
 // its axes the pass moves v and w at 5.8 TB/s.  Measured (GB300, whole H_up
-// pass): three orbitals at Ns = 18 17.4 -> 7.2 ms, two orbitals at Ns = 16
+// pass): three orbitals at Ns = 18 17.4 -> 7.5 ms, two orbitals at Ns = 16
 // 0.49 ms, against kernels that read an ELL table of H_up from L2 and gather
 // staged rows.  Tried and slower: persistent CTAs that prefetch the next item
 // (8.2 / 0.53 ms: fewer warps per SM), pairs of rows on packed FP32 FMAs (7.7 /

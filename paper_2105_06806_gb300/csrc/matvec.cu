@@ -481,8 +481,8 @@ static int fiber_shape(int g, int64_t w) {
 }
 
 // Products (ms) of the orbital-factorised pass with the H_dw pass against the
-// kernels it replaces in the tiled family: Norb=3 Ns=18 14.7 / 24.9, Norb=2
-// Ns=16 0.96 / 1.13, Norb=3 Ns=15 0.31 / 0.45, Norb=4 Ns=16 1.28 / 1.84; the
+// kernels it replaces in the tiled family: Norb=3 Ns=18 15.0 / 24.9, Norb=2
+// Ns=16 0.95 / 1.13, Norb=3 Ns=15 0.30 / 0.45, Norb=4 Ns=16 1.28 / 1.84; the
 // autotuner still compares the family with the element-parallel kernel.
 // Group size of the orbital-factorised product where the sector's FP32
 // block-major product can take it, else 0: one orbital has no factorisation,
