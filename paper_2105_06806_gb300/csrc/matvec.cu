@@ -1568,8 +1568,8 @@ static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st)
         else
           k_hv_rows<T, MODE, false><<<grid, HVS_THREADS, 0, st>>>(a);
       }
-    } else if (sizeof(T) == 8 && a.tb.small_chunk[L] > 1)
-      k_hv_small<T, MODE, sizeof(T) == 8><<<grid, HVS_THREADS, 0, st>>>(a);
+    } else if (a.tb.small_chunk[L] > 1)
+      k_hv_small<T, MODE, true><<<grid, HVS_THREADS, 0, st>>>(a);
     else
       k_hv_small<T, MODE, false><<<grid, HVS_THREADS, 0, st>>>(a);
   } else if (a.tb.fiber) {
