@@ -40,44 +40,24 @@ __device__ __forceinline__ double warp_sum(double x) {
   return x;
 }
 
-// Deterministic sums of n partials of each of N sets by one CTA, in every
-// thread: thread t adds the strided subsequences t, t+T, ... in order, then two
-// shuffle trees.  The chain of dependent FP64 additions is what this costs (a
-// second level summed by one thread, and one set after the other, took k_beta
-// of a chain 6.3 us, now 5.3).  red: N * 32 doubles.
-template <int N>
-__device__ void cta_sums(const double *const (&p)[N], int64_t n, double *red, double (&out)[N]) {
-  double s[N];
-#pragma unroll
-  for (int q = 0; q < N; ++q) s[q] = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x)
-#pragma unroll
-    for (int q = 0; q < N; ++q) s[q] += p[q][i];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-#pragma unroll
-  for (int q = 0; q < N; ++q) {
-    s[q] = warp_sum(s[q]);
-    if (lane == 0) red[q * 32 + wid] = s[q];
-  }
-  __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int q = 0; q < N; ++q) {
-      const double t = warp_sum(lane < nw ? red[q * 32 + lane] : 0.0);
-      __syncwarp();
-      if (lane == 0) red[q * 32] = t;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < N; ++q) out[q] = red[q * 32];
-  __syncthreads();
-}
+// Deterministic sum of n partials by one CTA: thread t adds the strided
+// subsequence t, t+T, ... in order, then a fixed tree.
 __device__ double cta_sum_parts(const double *p, int64_t n, double *red) {
-  const double *const ps[1] = {p};
-  double out[1];
-  cta_sums<1>(ps, n, red, out);
-  return out[0];
+  double s = 0.0;
+  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) s += p[i];
+  s = warp_sum(s);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane == 0) red[wid] = s;
+  __syncthreads();
+  double tot = 0.0;
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) tot += red[k];
+    red[0] = tot;
+  }
+  __syncthreads();
+  tot = red[0];
+  __syncthreads();
+  return tot;
 }
 
 template <typename T>
@@ -284,7 +264,7 @@ __device__ double lowest_eigenvalue(const double *a, const double *b, const doub
 // the product leaves the partials of <v_j, H v_j>; <v_j, v_{j-1}> comes from
 // the previous step's update (k_axpy_norm, k_beta).
 __global__ void k_alpha(LanczosState *st, const double *part, const int64_t nparts) {
-  __shared__ double red[32];
+  __shared__ double red[SCALAR_THREADS / 32];
   if (st->done) return;
   double s = cta_sum_parts(part, nparts, red);
   if (threadIdx.x == 0) {
@@ -395,17 +375,15 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_axpy_norm(LanczosState *st, T 
 // beta_{j+1}, scale, Ritz value and stop test.  The Ritz value is evaluated
 // at steps 1 and 2, at the scheduled steps (next_check) and at the last step.
 __global__ void k_beta(LanczosState *st, const double *part, int64_t nparts) {
-  __shared__ double red[64];
+  __shared__ double red[SCALAR_THREADS / 32];
   __shared__ int stop;
   // T_k, its squared off-diagonal, then (inverse iteration) pivots and y
   __shared__ double s_a[ED_MAX_LANCZOS], s_b[ED_MAX_LANCZOS], s_b2[ED_MAX_LANCZOS];
   __shared__ double s_rp[ED_MAX_LANCZOS], s_y[ED_MAX_LANCZOS];
   __shared__ double s_be, s_hint[2];
   if (st->done) return;
-  const double *const sets[2] = {part, part + nparts};
-  double sums[2];
-  cta_sums<2>(sets, nparts, red, sums);
-  const double s2 = sums[0], c2 = sums[1];  // ||w||^2, <w, v_j>
+  double s2 = cta_sum_parts(part, nparts, red);
+  const double c2 = cta_sum_parts(part + nparts, nparts, red);  // <w, v_j>
   const int j = st->j;
   // scalar work once, by thread 0 (FP64 is the slow pipe)
   if (threadIdx.x == 0) {
@@ -537,7 +515,7 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_norm2(const T *v, int64_t n, d
 // Initialise the recurrence state: v_0 = buffer 0 scaled by 1/||buffer 0||.
 __global__ void k_state_init(LanczosState *st, const double *part, int64_t nparts, int maxit,
                              double tol, int check_every, double check_growth) {
-  __shared__ double red[32];
+  __shared__ double red[SCALAR_THREADS / 32];
   double s = cta_sum_parts(part, nparts, red);
   if (threadIdx.x == 0) {
     st->j = 0;
@@ -732,7 +710,7 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_rq_parts(const double *psi, co
 }
 
 __global__ void k_rq_final(const double *part, int64_t nparts, double *out) {
-  __shared__ double red[32];
+  __shared__ double red[SCALAR_THREADS / 32];
   double a = cta_sum_parts(part, nparts, red);
   double c = cta_sum_parts(part + nparts, nparts, red);
   if (threadIdx.x == 0) {
@@ -764,7 +742,7 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_resid_parts(const double *psi,
 }
 
 __global__ void k_resid_final(const double *part, int64_t nparts, double *out) {
-  __shared__ double red[32];
+  __shared__ double red[SCALAR_THREADS / 32];
   double b = cta_sum_parts(part, nparts, red);
   if (threadIdx.x == 0) out[1] = sqrt(b / out[2]);
 }
@@ -813,11 +791,8 @@ struct Workspace {
   ~Workspace() { ed_dfree(mem, st); }
 };
 
-// CTAs of the streaming kernels: 8 elements per thread, 2 on sectors of a few
-// thousand elements, where a step is a chain of latencies
 static int64_t reduce_grid(int64_t n) {
-  const int64_t per = AXPY_THREADS * (n < (1 << 16) ? 2 : 8);
-  int64_t g = (n + per - 1) / per;
+  int64_t g = (n + AXPY_THREADS * 8 - 1) / (AXPY_THREADS * 8);
   return std::max<int64_t>(1, std::min<int64_t>(g, 152 * 8));
 }
 
