@@ -307,12 +307,13 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_axpy_norm(LanczosState *st, T 
   const T *v = basis ? basis[j] : bufs[j % 3];
   const T *prev = basis ? basis[j > 0 ? j - 1 : 0] : bufs[(j + 2) % 3];
   T *w = basis ? basis[j + 1] : bufs[(j + 1) % 3];
-  // the vectors' lazy scales are folded into the coefficients: 4 operations
-  // per element instead of 6 (FP64, where the update is bound by the FP64
-  // pipe: 136 -> 91 us at 1.18e7 elements, of which 65 us are HBM traffic)
+  // FP64 folds the vectors' lazy scales into the coefficients: 4 operations
+  // per element instead of 6 (the update is bound by the FP64 pipe: 136 -> 91
+  // us at 1.18e7 elements, of which 65 us are HBM traffic)
   const double sc = st->scale[j % 3], sc_prev = st->scale[(j + 2) % 3];
-  const T al = (T)(st->alpha[j] * sc);
-  const T be = (T)(st->beta[j] * sc_prev);
+  const T s_cur = (T)sc, s_prev = (T)sc_prev;
+  const T al = coef_of<T>(st->alpha[j], sc);
+  const T be = coef_of<T>(st->beta[j], sc_prev);
   // Block-major vectors are 16-byte aligned and their length is a multiple
   // of 4 elements: 16-byte accesses, one vector per thread and iteration.
   // Per-thread sums in T over at most FLUSH elements, then into FP64.
@@ -344,10 +345,11 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_axpy_norm(LanczosState *st, T 
       if (j > 0) VT::get(pv[i], pr);
 #pragma unroll
       for (int q = 0; q < NV; ++q) {
-        if (j > 0) x[q] = fmaT<T>(-be, pr[q], x[q]);
-        x[q] = fmaT<T>(-al, vi[q], x[q]);
+        const T vq = vec_of<T>(vi[q], s_cur);
+        if (j > 0) x[q] = fmaT<T>(-be, vec_of<T>(pr[q], s_prev), x[q]);
+        x[q] = fmaT<T>(-al, vq, x[q]);
         acc = fmaT<T>(x[q], x[q], acc);
-        cvv = fmaT<T>(x[q], vi[q], cvv);
+        cvv = fmaT<T>(x[q], vq, cvv);
       }
       wv[i] = VT::make(x);
       if (psi) {
@@ -368,7 +370,7 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_axpy_norm(LanczosState *st, T 
   const double totc = cta_sum<AXPY_THREADS>(cvvd, red[1]);
   if (threadIdx.x == 0) {
     part[blockIdx.x] = tot;
-    part[gridDim.x + blockIdx.x] = totc * sc;  // v_j = sc * (the vector read)
+    part[gridDim.x + blockIdx.x] = totc * fold_of<T>(s_cur);
   }
 }
 

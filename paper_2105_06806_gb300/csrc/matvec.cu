@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
   struct EpState {
     T *out;
     const T *prev;
-    T s_cur, beta_s, alpha_s, y_s;  // scale of v_j; beta, alpha, y times their vector's scale
+    T s_cur, s_prev, beta_s, alpha_s, y_s;  // scales of v_j, v_{j-1}; coefficients (see coef_of)
     int j;
   };
   __shared__ EpState ep_s;
@@ -974,8 +974,9 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
       }
       const double sc = st->scale[j % 3];
       e.s_cur = (T)sc;
-      e.beta_s = (T)(st->beta[j] * st->scale[(j + 2) % 3]);
-      e.alpha_s = MODE == HV_SECOND ? (T)(st->alpha[j] * sc) : T(0);
+      e.s_prev = (T)st->scale[(j + 2) % 3];
+      e.beta_s = coef_of<T>(st->beta[j], st->scale[(j + 2) % 3]);
+      e.alpha_s = MODE == HV_SECOND ? coef_of<T>(st->alpha[j], sc) : T(0);
       e.y_s = MODE == HV_SECOND ? (T)(st->y[j] * sc) : T(0);
       ep_s = e;
     }
@@ -1097,7 +1098,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
               if (i >= nrt || (!full && c >= nc)) continue;
               const T w1 = mul_t<T>(acc[u][i], s_cur);
               acc[u][i] = w1;
-              dot = fma_t<T>(xr[i], w1, dot);
+              dot = fma_t<T>(vec_of<T>(xr[i], s_cur), w1, dot);
             }
           }
 #pragma unroll
@@ -1116,7 +1117,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
           continue;
         }
         // second pass: the step's scalars, read from shared memory once per tile
-        const T s_cur = ep.s_cur, beta_s = ep.beta_s;
+        const T s_cur = ep.s_cur, s_prev = ep.s_prev, beta_s = ep.beta_s;
         const T alpha_s = ep.alpha_s, y_s = ep.y_s;
         const T *const prev = ep.prev;
         const bool has_prev = ep.j > 0;
@@ -1142,8 +1143,8 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
             if (!full && c >= nc) continue;
             const T xv = staged ? smq[(size_t)stage_pos(c, ncp >> 2) * RT + i] : g[rb + u];
             T w1 = mul_t<T>(acc[u][i], s_cur);
-            if (has_prev) w1 = fma_t<T>(-beta_s, pv[u], w1);
-            res[u] = fma_t<T>(-alpha_s, xv, w1);
+            if (has_prev) w1 = fma_t<T>(-beta_s, vec_of<T>(pv[u], s_prev), w1);
+            res[u] = fma_t<T>(-alpha_s, vec_of<T>(xv, s_cur), w1);
             a.psi[rb + u] = fma_t<T>(y_s, xv, a.psi[rb + u]);
           }
           if (vec) {
@@ -1158,9 +1159,8 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
     }
   }
   if (MODE == HV_LANCZOS && !PASSA) {
-    // <v_j, w1> with v_j = s_cur * (the vector read)
     double smv = block_sum<T>((double)dot, red);
-    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * (double)ep_s.s_cur;
+    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * fold_of<T>(ep_s.s_cur);
   }
 }
 
@@ -1185,7 +1185,7 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
   __shared__ int32_t s_dn[DW_ROWS];
   const HvTables<T> &tb = a.tb;
   int j = 0;
-  T s_cur = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
+  T s_cur = T(1), s_prev = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
   const T *g;
   const T *prev = nullptr;
   T *out;
@@ -1207,8 +1207,9 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
     }
     s_cur = (T)st->scale[m3];
     if (MODE == HV_SECOND) {
-      beta_s = (T)(st->beta[j] * st->scale[(j + 2) % 3]);
-      alpha_s = (T)(st->alpha[j] * st->scale[m3]);
+      s_prev = (T)st->scale[(j + 2) % 3];
+      beta_s = coef_of<T>(st->beta[j], st->scale[(j + 2) % 3]);
+      alpha_s = coef_of<T>(st->alpha[j], st->scale[m3]);
       y_s = (T)(st->y[j] * st->scale[m3]);
     }
   }
@@ -1277,12 +1278,12 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
           const T x = g[gi];
           T w1 = mul_t<T>(acc[i][u], s_cur);
           if (MODE == HV_SECOND && j > 0)  // the Lanczos step does this in its update
-            w1 = fma_t<T>(-beta_s, prev[gi], w1);
+            w1 = fma_t<T>(-beta_s, vec_of<T>(prev[gi], s_prev), w1);
           if (MODE == HV_LANCZOS) {
             out[gi] = w1;
-            dot = fma_t<T>(x, w1, dot);
+            dot = fma_t<T>(vec_of<T>(x, s_cur), w1, dot);
           } else {
-            out[gi] = fma_t<T>(-alpha_s, x, w1);
+            out[gi] = fma_t<T>(-alpha_s, vec_of<T>(x, s_cur), w1);
             a.psi[gi] = fma_t<T>(y_s, x, a.psi[gi]);
           }
         }
@@ -1291,7 +1292,7 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
   }
   if (MODE == HV_LANCZOS) {
     const double smv = cta_sum<DW_THREADS>(dotd + (double)dot, red);
-    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * (double)s_cur;  // v_j = s_cur x
+    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * fold_of<T>(s_cur);
   }
 }
 
@@ -1305,7 +1306,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
   __shared__ double red[MODE == HV_LANCZOS ? HVS_THREADS : 1];
   const HvTables<T> &tb = a.tb;
   int j = 0;
-  T s_cur = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
+  T s_cur = T(1), s_prev = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
   const T *g;
   const T *prev = nullptr;
   T *out;
@@ -1327,8 +1328,9 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
     }
     s_cur = (T)st->scale[m3];
     if (MODE == HV_SECOND) {
-      beta_s = (T)(st->beta[j] * st->scale[(j + 2) % 3]);
-      alpha_s = (T)(st->alpha[j] * st->scale[m3]);
+      s_prev = (T)st->scale[(j + 2) % 3];
+      beta_s = coef_of<T>(st->beta[j], st->scale[(j + 2) % 3]);
+      alpha_s = coef_of<T>(st->alpha[j], st->scale[m3]);
       y_s = (T)(st->y[j] * st->scale[m3]);
     }
   }
@@ -1367,12 +1369,12 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
       } else {
         T w1 = mul_t<T>(acc, s_cur);
         if (MODE == HV_SECOND && j > 0)  // the Lanczos step does this in its update
-          w1 = fma_t<T>(-beta_s, prev[gi], w1);
+          w1 = fma_t<T>(-beta_s, vec_of<T>(prev[gi], s_prev), w1);
         if (MODE == HV_LANCZOS) {
           out[gi] = w1;
-          dot = fma_t<T>(x, w1, dot);
+          dot = fma_t<T>(vec_of<T>(x, s_cur), w1, dot);
         } else {
-          out[gi] = fma_t<T>(-alpha_s, x, w1);
+          out[gi] = fma_t<T>(-alpha_s, vec_of<T>(x, s_cur), w1);
           a.psi[gi] = fma_t<T>(y_s, x, a.psi[gi]);
         }
       }
@@ -1380,7 +1382,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
   }
   if (MODE == HV_LANCZOS) {
     const double smv = cta_sum<HVS_THREADS>(dot_sum + (double)dot, red);
-    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * (double)s_cur;  // v_j = s_cur x
+    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * fold_of<T>(s_cur);
   }
 }
 
@@ -1390,7 +1392,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_rows(HvLaunch<T> a) {
   __shared__ double red[MODE == HV_LANCZOS ? HVS_THREADS : 1];
   const HvTables<T> &tb = a.tb;
   int j = 0;
-  T s_cur = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
+  T s_cur = T(1), s_prev = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
   const T *g;
   const T *prev = nullptr;
   T *out;
@@ -1412,8 +1414,9 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_rows(HvLaunch<T> a) {
     }
     s_cur = (T)st->scale[m3];
     if (MODE == HV_SECOND) {
-      beta_s = (T)(st->beta[j] * st->scale[(j + 2) % 3]);
-      alpha_s = (T)(st->alpha[j] * st->scale[m3]);
+      s_prev = (T)st->scale[(j + 2) % 3];
+      beta_s = coef_of<T>(st->beta[j], st->scale[(j + 2) % 3]);
+      alpha_s = coef_of<T>(st->alpha[j], st->scale[m3]);
       y_s = (T)(st->y[j] * st->scale[m3]);
     }
   }
@@ -1470,12 +1473,12 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_rows(HvLaunch<T> a) {
       } else {
         T w1 = mul_t<T>(acc[q], s_cur);
         if (MODE == HV_SECOND && j > 0)  // the Lanczos step does this in its update
-          w1 = fma_t<T>(-beta_s, prev[gi], w1);
+          w1 = fma_t<T>(-beta_s, vec_of<T>(prev[gi], s_prev), w1);
         if (MODE == HV_LANCZOS) {
           out[gi] = w1;
-          dot = fma_t<T>(x[q], w1, dot);
+          dot = fma_t<T>(vec_of<T>(x[q], s_cur), w1, dot);
         } else {
-          out[gi] = fma_t<T>(-alpha_s, x[q], w1);
+          out[gi] = fma_t<T>(-alpha_s, vec_of<T>(x[q], s_cur), w1);
           a.psi[gi] = fma_t<T>(y_s, x[q], a.psi[gi]);
         }
       }
@@ -1483,7 +1486,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_rows(HvLaunch<T> a) {
   }
   if (MODE == HV_LANCZOS) {
     const double smv = cta_sum<HVS_THREADS>(dot_sum + (double)dot, red);
-    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * (double)s_cur;  // v_j = s_cur x
+    if (threadIdx.x == 0) a.part[blockIdx.x] = smv * fold_of<T>(s_cur);
   }
 }
 

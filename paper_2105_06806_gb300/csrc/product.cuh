@@ -65,6 +65,25 @@ struct HvLaunch {
   int64_t slice = 0;  // HV_SLICED: grid row y works on v + y * slice, w + y * slice
 };
 
+// Lazy scales of the Lanczos vectors (v_j = scale * the stored vector).  FP64, bound
+// by its pipe, folds the scale into the recurrence's coefficients; FP32 scales
+// each element before it is used, which keeps its rounding that of normalised
+// vectors and costs nothing beside the memory traffic.
+template <typename T>
+__device__ __forceinline__ T vec_of(T x, T scale) {
+  if constexpr (sizeof(T) == 8) return x;
+  else return mul_t<T>(x, scale);
+}
+template <typename T>
+__device__ __forceinline__ T coef_of(double c, double scale) {
+  return (T)(sizeof(T) == 8 ? c * scale : c);
+}
+// what a sum over vec_of elements still has to be multiplied with
+template <typename T>
+__device__ __forceinline__ double fold_of(T scale) {
+  return sizeof(T) == 8 ? (double)scale : 1.0;
+}
+
 // Sum over a CTA of NT threads (fixed order), in thread 0 of the first warp:
 // the values cross shared memory and one warp adds them.  A shuffle tree in
 // every warp would cost each thread 5 FP64 additions, as much FP64 issue as a
