@@ -24,6 +24,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "dispatch.h"
 #include "product.cuh"
 
 // Register tile: 4 consecutive columns x RT rows; the RT rows of one column
@@ -123,20 +124,13 @@ constexpr int HVS_THREADS = 256;
 #ifndef EDGB_SMALL_LANCZOS_PARTS
 #define EDGB_SMALL_LANCZOS_PARTS (1 << 13)
 #endif
-// Rows per thread: in FP32 above 2^22 elements a thread takes one column of 4
-// consecutive rows (k_hv_rows), which share the column's tables and H_up
-// entries and have their gathers in flight together (Norb=1 Ns=14 145 -> 113
-// us, Norb=5 Ns=14 509 -> 367 us).  Smaller sectors need the threads (1-2%
-// slower at 10^6 elements), and FP64 is bound by its pipe (5.80 against 5.57 ms
-// at Norb=2 Ns=16).
-constexpr int HVS_ROWS = 4;
 static bool small_rows_of(ed_sector s, int elem) {
-  return elem == 4 && s->bdim > (int64_t)1 << 22;
+  return ed_takes_rows(elem, s->sp[1].dim, s->bstride);
 }
 // CTAs of 256 elements (columns of rows), chunks of them per CTA, CTAs launched
 static int64_t small_blocks_of(ed_sector s, int elem) {
-  const int64_t rows = small_rows_of(s, elem) ? HVS_ROWS : 1;
-  const int64_t units = (s->sp[1].dim + rows - 1) / rows * s->bstride;
+  const int64_t units =
+      small_rows_of(s, elem) ? ed_rows_units(s->sp[1].dim, s->bstride) : s->bdim;
   return (units + HVS_THREADS - 1) / HVS_THREADS;
 }
 static int64_t small_chunk_of(ed_sector s, int elem, bool lanczos) {
@@ -1386,7 +1380,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_small(HvLaunch<T> a) {
   }
 }
 
-// The same product, one thread per column of HVS_ROWS rows (see small_rows_of).
+// The same product, one thread per column of HVS_ROWS rows (see ed_takes_rows).
 template <typename T, int MODE, bool CHUNKED>
 __global__ void __launch_bounds__(HVS_THREADS) k_hv_rows(HvLaunch<T> a) {
   __shared__ double red[MODE == HV_LANCZOS ? HVS_THREADS : 1];
@@ -1423,8 +1417,7 @@ __global__ void __launch_bounds__(HVS_THREADS) k_hv_rows(HvLaunch<T> a) {
   const int64_t stride = tb.stride;
   T dot = T(0);
   double dot_sum = 0.0;  // the per-thread sum, flushed from T every 16 elements
-  // units of work: (group of HVS_ROWS rows, padded column); fewer than 2^32
-  const int64_t units = (tb.ddw + HVS_ROWS - 1) / HVS_ROWS * stride;
+  const int64_t units = ed_rows_units(tb.ddw, stride);  // at most 2^32 (ed_takes_rows)
   const int K = CHUNKED ? tb.small_chunk[MODE == HV_LANCZOS] : 1;
   for (int k = 0; k < K; ++k) {
     const int64_t u = ((int64_t)blockIdx.x * K + k) * HVS_THREADS + threadIdx.x;
