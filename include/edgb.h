@@ -607,6 +607,10 @@ ed_status ed_residual_noalloc(ed_sector s, const double *d_psi, int64_t n, doubl
  * NULL output. */
 ed_status ed_memory_trim(int64_t keep_bytes);
 ed_status ed_memory_cached(int64_t *reserved, int64_t *used);
+/* Test hook: the after-th following device allocation of the calling host
+ * thread (1: the next one) fails with ED_ERR_OOM; 0 clears a pending failure.
+ * ED_ERR_ARG on a negative count. */
+ed_status ed_inject_alloc_failure(int32_t after);
 
 const char *ed_status_string(ed_status st);
 const char *ed_last_error(void);

@@ -35,7 +35,7 @@ EXPORTED = [
     "ed_server_create", "ed_submit", "ed_poll", "ed_wait", "ed_server_destroy",
     "ed_server_inject_alloc_failure", "ed_batch_stats", "ed_residual_noalloc", "ed_status_string",
     "ed_last_error",
-    "ed_kernel_launches", "ed_memory_trim", "ed_memory_cached",
+    "ed_kernel_launches", "ed_memory_trim", "ed_memory_cached", "ed_inject_alloc_failure",
 ]
 
 
@@ -177,6 +177,7 @@ def lib():
             "ed_batch_stats": [C.POINTER(i64), C.POINTER(i64), C.POINTER(i64)],
             "ed_memory_trim": [i64],
             "ed_memory_cached": [C.POINTER(i64), C.POINTER(i64)],
+            "ed_inject_alloc_failure": [i32],
             "ed_gf_lanczos_z": [vp, C.c_int, vp, C.c_double, i32, i32, i32, vp, i32, vp,
                                 C.POINTER(ed_gf_info), vp],
             "ed_sigma": [C.POINTER(ed_model), i32, i32, vp, i32, vp, vp, vp],
@@ -410,6 +411,12 @@ def memory_cached():
     r, u = C.c_int64(), C.c_int64()
     _check(lib().ed_memory_cached(C.byref(r), C.byref(u)), "ed_memory_cached")
     return r.value, u.value
+
+
+def inject_alloc_failure(after):
+    """The after-th following device allocation of this thread fails; 0 clears
+    (ed_inject_alloc_failure, a test hook)."""
+    _check(lib().ed_inject_alloc_failure(int(after)), "ed_inject_alloc_failure")
 
 
 def batch_stats():

@@ -490,7 +490,7 @@ static int fiber_group(ed_sector s) {
 }
 
 static ed_status build_dw_items(ed_sector s, ItemList &il, int elem, cudaStream_t cs) {
-  if (il.d_ditems || (!il.fiber && !two_pass_wanted(s, elem))) return ED_OK;
+  if (!il.fiber && !two_pass_wanted(s, elem)) return ED_OK;
   const std::vector<int64_t> &ob_dw = s->bi[1].offset, &ob_up = s->bi[0].offset;
   std::vector<DwItem> items;
   for (size_t bd = 0; bd + 1 < ob_dw.size(); ++bd) {
@@ -517,7 +517,6 @@ static ed_status build_dw_items(ed_sector s, ItemList &il, int elem, cudaStream_
   }
   il.nditems = (int64_t)items.size();
   il.d_ditems = d;
-  s->device_bytes += (int64_t)(items.size() * sizeof(DwItem));
   return ED_OK;
 }
 
@@ -751,42 +750,39 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
                                (int32_t)nc, (int32_t)op_up[bu], deg, eoff, ncp});
     }
   }
-  HvItem *d_items = nullptr;
-  ED_TRY(ed_dmalloc((void **)&d_items, std::max<size_t>(items.size(), 1) * sizeof(HvItem), cs,
-                    "work items"));
+  ItemList t;
+  t.nitems = (int64_t)items.size();
+  t.smem = smem;
+  t.fiber = fiber;
+  t.fib = fib;
+  for (int k = 0; k < FIBER_SHAPES; ++k) t.nfib[k] = nfib[k];
+  ed_status rs = ed_dmalloc((void **)&t.d_items, std::max<size_t>(items.size(), 1) * sizeof(HvItem),
+                            cs, "work items");
+  if (rs == ED_OK && !fib.empty())
+    rs = ed_dmalloc((void **)&t.d_fib, fib.size() * sizeof(FibBlock), cs, "work items");
   cudaError_t e = cudaSuccess;
-  if (!items.empty())
-    e = cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(HvItem),
+  if (rs == ED_OK && !items.empty())
+    e = cudaMemcpyAsync(t.d_items, items.data(), items.size() * sizeof(HvItem),
                         cudaMemcpyHostToDevice, cs);
-  FibBlock *d_fib = nullptr;
-  if (!fib.empty() && e == cudaSuccess) {
-    const ed_status fs = ed_dmalloc((void **)&d_fib, fib.size() * sizeof(FibBlock), cs, "work items");
-    if (fs != ED_OK) {
-      ed_dfree(d_items, cs);
-      return fs;
-    }
-    e = cudaMemcpyAsync(d_fib, fib.data(), fib.size() * sizeof(FibBlock), cudaMemcpyHostToDevice, cs);
-  }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
-  if (e != cudaSuccess) {
+  if (rs == ED_OK && e == cudaSuccess && !fib.empty())
+    e = cudaMemcpyAsync(t.d_fib, fib.data(), fib.size() * sizeof(FibBlock), cudaMemcpyHostToDevice,
+                        cs);
+  if (rs == ED_OK && e == cudaSuccess) e = cudaStreamSynchronize(cs);
+  if (rs == ED_OK && e != cudaSuccess) {
     ed_set_cuda_error(e, "work items upload", __FILE__, __LINE__);
-    ed_dfree(d_items, cs);
-    ed_dfree(d_fib, cs);
-    return ED_ERR_CUDA;
+    rs = ED_ERR_CUDA;
   }
-  // published only once complete
-  il.nitems = (int64_t)items.size();
-  il.smem = smem;
-  il.fiber = fiber;
-  il.fib = fib;
-  il.d_fib = d_fib;
-  for (int k = 0; k < FIBER_SHAPES; ++k) il.nfib[k] = nfib[k];
-  il.d_items = d_items;
-  s->device_bytes += (int64_t)(items.size() * sizeof(HvItem));
-  if (layout == 1) {
-    ED_TRY(build_dw_items(s, il, elem, cs));
-    ED_TRY(decide_kernel(s, elem, cs));
+  if (rs == ED_OK && layout == 1) rs = build_dw_items(s, t, elem, cs);
+  if (rs != ED_OK) {
+    ed_dfree(t.d_items, cs);
+    ed_dfree(t.d_fib, cs);
+    return rs;
   }
+  // published only once complete, the H_dw list with the others
+  il = t;
+  s->device_bytes += (int64_t)(items.size() * sizeof(HvItem) + fib.size() * sizeof(FibBlock) +
+                               t.nditems * sizeof(DwItem));
+  if (layout == 1) ED_TRY(decide_kernel(s, elem, cs));
   return ED_OK;
 }
 

@@ -32,6 +32,9 @@ constexpr int kMaxDevices = 64;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {nullptr};
 
+// countdown of ed_inject_alloc_failure, per host thread (0: off)
+thread_local int32_t t_fail_after = 0;
+
 std::mutex g_flag_mu;
 std::vector<int32_t *> g_free_flags;
 constexpr int kFlagStride = 16;   // one 64-byte line per flag
@@ -90,6 +93,10 @@ struct ThreadStreams {
 
 ed_status ed_dmalloc(void **p, size_t bytes, cudaStream_t st, const char *what) {
   *p = nullptr;
+  if (t_fail_after > 0 && --t_fail_after == 0) {
+    ed_set_error_msg("device allocation failed (injected)");
+    return ED_ERR_OOM;
+  }
   cudaMemPool_t pool = nullptr;
   ED_TRY(device_pool(&pool));
   cudaError_t e = cudaMallocFromPoolAsync(p, bytes > 0 ? bytes : 1, pool, st);
@@ -131,6 +138,12 @@ extern "C" ed_status ed_memory_trim(int64_t keep_bytes) {
   cudaMemPool_t pool = nullptr;
   ED_TRY(device_pool(&pool));
   ED_TRY_CUDA(cudaMemPoolTrimTo(pool, (size_t)keep_bytes));
+  return ED_OK;
+}
+
+extern "C" ed_status ed_inject_alloc_failure(int32_t after) {
+  if (after < 0) return ED_ERR_ARG;
+  t_fail_after = after;
   return ED_OK;
 }
 

@@ -1,0 +1,62 @@
+"""Failed device allocations (injected on the host, one at a time): the call
+either reports ED_ERR_OOM or does without the memory, and the sector works as
+if nothing had happened once memory is there again."""
+import pytest
+import torch
+
+from workloads import make_model
+
+pytestmark = pytest.mark.gpu
+
+DT = {"fp32": torch.float32, "fp64": torch.float64}
+
+
+def _vec(n, dt, seed=1):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.rand(n, device="cuda", dtype=dt, generator=g) - 0.5
+
+
+def _failures(ed, call, most=40):
+    """Runs `call(n)` (which makes its n-th allocation fail) for n = 1, 2, .. until
+    one needs fewer allocations; returns the number of calls that met a failure."""
+    for n in range(1, most):
+        try:
+            met = call(n)
+        finally:
+            ed.inject_alloc_failure(0)
+        if not met:
+            return n - 1
+    raise AssertionError("a call allocates more than expected")
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("case", [(2, 6, 5, 4), (1, 11, 6, 5), (2, 3, 4, 4)])
+def test_product_after_a_failed_allocation(ed, case, prec):
+    """Every allocation of a sector's first block-major product fails once; the
+    next product on the same sector gives w bit for bit."""
+    norb, nbath, nup, ndw = case
+    m = make_model(norb, nbath, U=2.0, Jh=0.3 * (norb > 1), seed=4)
+    ref = ed.Sector(m, nup, ndw)
+    v = torch.empty(ref.blocked_dim, device="cuda", dtype=DT[prec])
+    ed.permute(ref, _vec(ref.dim, DT[prec]), v, True, prec)
+    want = torch.zeros_like(v)
+    ed.matvec_blocked(ref, v, want, prec)
+    ref.free()
+
+    def call(n):
+        s = ed.Sector(m, nup, ndw)
+        ed.inject_alloc_failure(n)
+        failed = False
+        try:
+            ed.matvec_blocked(s, v, torch.zeros_like(v), prec)
+        except ed.EDError as e:
+            assert e.status == ed.ED_ERR_OOM
+            failed = True
+        ed.inject_alloc_failure(0)
+        w = torch.zeros_like(v)
+        ed.matvec_blocked(s, v, w, prec)
+        assert torch.equal(w, want)
+        s.free()
+        return failed
+
+    assert _failures(ed, call) >= 2
