@@ -141,7 +141,16 @@ ed_status ed_sector_free(ed_sector s);
  *          + sum_k H_up[c,k] v[r,k] + sum_k H_dw[r,k] v[k,c].
  * d_v, d_w: device arrays of n = D elements, double for ED_FP64, float for
  * ED_FP32 / ED_FP32_POLISH; must not overlap.  ED_ERR_ARG when n != D.
- * Asynchronous on `stream`. */
+ * Asynchronous on `stream`.
+ *
+ * Large FP32 sectors of several orbitals go through block-major order where
+ * that is the faster way (from 2^25 elements with two or three orbitals, 2^27
+ * with four; from 2^20 where ed_sector_set_kernel pinned the tiled family),
+ * in a scratch of two vectors that returns to the library's pool
+ * (ed_memory_trim).  Without memory for it, and on a stream under
+ * capture, the sector-order kernel serves the call: the same sum of the same
+ * terms in another order, so w can differ in its last bits between two such
+ * calls (about 1e-7 of sum_k |H_ik v_k|). */
 ed_status ed_matvec(ed_sector s, ed_precision prec, const void *d_v, void *d_w, int64_t n,
                     void *stream);
 
@@ -203,7 +212,7 @@ ed_status ed_sector_blocked_kernel(ed_sector s, ed_precision prec, int32_t *kern
  * kernel for one sector and precision: ED_KERNEL_ELEMENTWISE or the tiled
  * family (ED_KERNEL_TILED, or
  * ED_KERNEL_TWO_PASS where the block sizes call for two passes); other
- * requests give ED_ERR_UNSUPPORTED.  All kernels compute the same w = H v bit
+ * requests give ED_ERR_UNSUPPORTED.  ed_matvec follows a pin as described there.  All kernels compute the same w = H v bit
  * for bit; Lanczos runs differ only in the summation order of <v, w>. */
 ed_status ed_sector_tune_info(ed_sector s, ed_precision prec, int32_t *kernel, double *host_ms);
 ed_status ed_sector_set_kernel(ed_sector s, ed_precision prec, int32_t kernel);

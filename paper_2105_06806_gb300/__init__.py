@@ -383,7 +383,10 @@ def _matvec(f, name, sector, v, w, precision, stream):
 
 
 def matvec(sector: Sector, v, w, precision="fp64", stream=None):
-    """w = H v for device tensors (float64 for fp64, float32 otherwise)."""
+    """w = H v for device tensors (float64 for fp64, float32 otherwise).  Large FP32
+    products of several orbitals can go through block-major order in a scratch of
+    the library's pool; without memory for it, or under stream capture, w can
+    differ in its last bits (ed_matvec in include/edgb.h)."""
     _matvec(lib().ed_matvec, "ed_matvec", sector, v, w, precision, stream)
 
 

@@ -24,3 +24,24 @@ constexpr bool ed_takes_rows(int elem, int64_t ddw, int64_t stride) {
   return elem == 4 && ddw * stride > (int64_t)1 << 22 &&
          ed_rows_units(ddw, stride) <= (int64_t)1 << 32;
 }
+
+// Sector-order FP32 product through block-major order (two permutations and
+// the orbital-factorised product in a scratch pair of vectors) instead of the
+// sector-order kernel, whose H_up hops gather across whole CSR rows.  Measured
+// on every sector within two electrons of half filling, sector-order kernel /
+// detour in us: two orbitals at Ns=16 1019 / 751 to 2724 / 1950 (9 sectors of
+// 9 faster), three at Ns=15 from 2^25 elements 714 / 570; below 2^25 elements
+// between 0.85 and 1.15 times, and mostly slower (Norb=2 Ns=14 (7,7) 146 / 158,
+// Norb=3 Ns=15 (5,7) 257 / 269); four orbitals 2542 / 2420 from 2^27
+// elements, below that 0.95 to 1.1 times; five orbitals 704 / 840.
+// group: levels of an orbital group, 0 where the factorised product does not
+// apply; pinned: the kernel the caller chose for the block-major layout (0 the
+// tiled family, which is then taken from 2^20 elements on, 1 element-parallel,
+// -1 none).
+constexpr int64_t ED_PERMUTE_MIN = (int64_t)1 << 20;
+constexpr int64_t ed_permute_scratch(int64_t bdim) { return 2 * bdim * (int64_t)sizeof(float); }
+constexpr bool ed_takes_permuted(int norb, int group, int64_t dim, int pinned) {
+  if (group == 0 || dim < ED_PERMUTE_MIN || pinned == 1) return false;
+  if (pinned == 0) return true;
+  return norb <= 3 ? dim >= (int64_t)1 << 25 : norb == 4 && dim >= (int64_t)1 << 27;
+}

@@ -199,7 +199,7 @@ struct ed_sector_s {
   // block-major product kernel per precision [FP32, FP64]: -1 undecided,
   // 0 tiled (one- or two-pass), 1 element-parallel; pinned or autotuned
   int8_t hv_kernel[2] = {-1, -1};
-  bool hv_pinned[2] = {false, false};
+  bool hv_pinned[2] = {false, false};  // chosen by ed_sector_set_kernel
   double tune_ms[2][2] = {{-1.0, -1.0}, {-1.0, -1.0}};  // [precision][tiled, element-parallel]
   NdTables nd[2];          // [layout]; empty when J_X = J_P = 0
   double *W = nullptr;     // [2^norb][2^norb]

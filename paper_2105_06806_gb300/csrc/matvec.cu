@@ -1633,20 +1633,15 @@ template ed_status ed_launch_hv<double>(ed_sector, const HvTables<double> &, int
                                         double *, int64_t *, cudaStream_t, double *const *, int,
                                         int64_t);
 
-// Sector-order FP32 product through block-major order: both permutations and
-// the orbital-factorised product in a scratch pair of vectors.  From
-// EDGB_PERMUTE_MIN elements this beats the sector-order kernel, whose H_up
-// hops gather across whole CSR rows (Norb=2 Ns=14 (5,6): 88
-// against 97 us, Norb=2 Ns=16 1.93 against 2.72 ms).
-// *done = false: not taken (the kernel choice, no memory for the scratch, or a
-// stream under capture, where the scratch would become part of the graph).
-#ifndef EDGB_PERMUTE_MIN
-#define EDGB_PERMUTE_MIN (1 << 20)
-#endif
+// Sector-order FP32 product through block-major order (see ed_takes_permuted).
+// *done = false: not taken (the rule, no memory for the scratch, or a stream
+// under capture, where the scratch would become part of the graph).
 static ed_status matvec_permuted(ed_sector s, const float *v, float *w, cudaStream_t st,
                                  bool *done) {
   *done = false;
-  if (s->mp.norb < 2 || s->dim < (int64_t)EDGB_PERMUTE_MIN) return ED_OK;
+  if (s->mp.norb < 2 || s->dim < ED_PERMUTE_MIN) return ED_OK;
+  const int pinned = s->hv_pinned[0] ? s->hv_kernel[0] : -1;
+  if (!ed_takes_permuted(s->mp.norb, fiber_group(s), s->dim, pinned)) return ED_OK;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
@@ -1655,10 +1650,10 @@ static ed_status matvec_permuted(ed_sector s, const float *v, float *w, cudaStre
   // both layouts' work lists, so that a later call under capture builds nothing
   ED_TRY(ed_build_items(s, 0, 4));
   ED_TRY(ed_build_items(s, 1, 4));
-  const HvTables<float> tb = ed_hv_tables<float>(s, 1);
-  if (!tb.fiber || tb.small_cols) return ED_OK;
+  HvTables<float> tb = ed_hv_tables<float>(s, 1);
+  tb.small_cols = nullptr;  // the factorised product, whatever the tuner chose
   void *mem = nullptr;
-  if (ed_dmalloc(&mem, 2 * s->bdim * sizeof(float), st, "permuted product") != ED_OK) {
+  if (ed_dmalloc(&mem, ed_permute_scratch(s->bdim), st, "permuted product") != ED_OK) {
     cudaGetLastError();
     ed_set_error_msg("");
     return ED_OK;
@@ -1762,6 +1757,7 @@ extern "C" ed_status ed_sector_set_kernel(ed_sector s, ed_precision prec, int32_
       return ED_ERR_UNSUPPORTED;
     }
     s->hv_kernel[e] = 1;
+    s->hv_pinned[e] = true;
   } else if (kernel == ED_KERNEL_TILED || kernel == ED_KERNEL_TWO_PASS) {
     // the tiled family: one or two passes as the sector's size decides
     if ((kernel == ED_KERNEL_TWO_PASS) != two_pass_wanted(s, e ? 8 : 4)) {
@@ -1769,6 +1765,7 @@ extern "C" ed_status ed_sector_set_kernel(ed_sector s, ed_precision prec, int32_
       return ED_ERR_UNSUPPORTED;
     }
     s->hv_kernel[e] = 0;
+    s->hv_pinned[e] = true;
   } else {
     return ED_ERR_ARG;
   }

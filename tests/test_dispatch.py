@@ -43,3 +43,24 @@ def test_rows_kernel_within_its_32_bit_units(tmp_path):
         if g:  # the largest unit's row and column survive the 32-bit division
             u = units(d, s) - 1
             assert ((u & 0xffffffff) // s, (u & 0xffffffff) % s) == (u // s, u % s)
+
+
+def test_sector_order_detour_rule(tmp_path):
+    """The sector-order FP32 product goes through block-major order only where that was
+    measured faster, and follows a pinned kernel."""
+    cases = [  # norb, group, dim, bdim, pinned, want
+        (2, 7, 11778624, 11806080, -1, 0),      # Norb=2 Ns=14 (7,7): slower
+        (2, 8, 165636900, 165791340, -1, 1),    # Norb=2 Ns=16 (8,8)
+        (3, 5, 41409225, 41460705, -1, 1),      # Norb=3 Ns=15 (7,7)
+        (3, 5, 15030015, 15100000, -1, 0),
+        (4, 4, 165636900, 166000000, -1, 1), (4, 4, 102951200, 103200000, -1, 0),
+        (5, 3, 41409225, 41900000, -1, 0),      # five orbitals: never faster
+        (2, 0, 2363904400, 2364000000, -1, 0),  # groups the factorised product does not take
+        (2, 8, 1 << 25, 1 << 25, -1, 1), (2, 8, (1 << 25) - 1, 1 << 25, -1, 0),
+        (4, 4, 1 << 27, 1 << 27, -1, 1), (4, 4, (1 << 27) - 1, 1 << 27, -1, 0),
+        (2, 7, 6012006, 6030000, 0, 1), (2, 7, (1 << 20) - 1, 1 << 20, 0, 0),  # tiled pinned
+        (5, 3, 1 << 20, 1 << 20, 0, 1), (2, 8, 165636900, 165791340, 1, 0),    # pinned
+    ]
+    got = _run(tmp_path, "\n".join('printf("%%d\\n", (int)ed_takes_permuted(%d, %d, %dLL, %d));'
+                                   % (c[0], c[1], c[2], c[4]) for c in cases))
+    assert got == [c[5] for c in cases]
