@@ -671,26 +671,17 @@ static void item_shape(int64_t nc, int elem, int RT, int threads, int64_t *rows,
 
 // Work items, ordered dw block by dw block, up block by up block, rows
 // ascending: while one block pair is processed, its |dw block| x |up block|
-// slice of v is the L2 working set of the H_dw reads.
-ed_status ed_build_items(ed_sector s, int layout, int elem) {
+// slice of v is the L2 working set of the H_dw reads.  Block-major items other
+// than the orbital-factorised product's read the ELL table's shape.
+static ed_status build_list(ed_sector s, int layout, int elem, cudaStream_t cs) {
   ItemList &il = s->items[layout][elem == 8 ? 1 : 0];
   if (il.d_items) return ED_OK;
-  // built once per sector on this thread's private stream, complete on return
-  ed_status ps = ED_OK;
-  cudaStream_t cs = ed_private_stream(&ps);
-  if (ps != ED_OK) return ps;
   std::vector<int64_t> ob_up, ob_dw, op_up;
   if (layout == 0) {
     ob_up = {0, s->sp[0].dim};
     op_up = ob_up;
     ob_dw = {0, s->sp[1].dim};
   } else {
-    // the orbital-factorised product reads no table of H_up: where the shape is
-    // known to take it, the ELL table waits until something else needs it
-    if (!(elem == 4 && fiber_group(s) && tuned_tiled(s, elem))) {
-      ED_TRY(ed_build_ell(s, cs));
-      ED_TRY(build_small_cols(s, cs));
-    }
     ob_up = s->bi[0].offset;
     op_up = s->up_off_pad;
     ob_dw = s->bi[1].offset;
@@ -782,8 +773,29 @@ ed_status ed_build_items(ed_sector s, int layout, int elem) {
   il = t;
   s->device_bytes += (int64_t)(items.size() * sizeof(HvItem) + fib.size() * sizeof(FibBlock) +
                                t.nditems * sizeof(DwItem));
-  if (layout == 1) ED_TRY(decide_kernel(s, elem, cs));
   return ED_OK;
+}
+
+// Everything a product in this layout and precision needs, built once per
+// sector on this thread's private stream, complete on return.
+static bool items_ready(ed_sector s, int layout, int elem) {
+  const int e = elem == 8 ? 1 : 0;
+  return s->items[layout][e].d_items && (layout == 0 || s->hv_kernel[e] >= 0);
+}
+ed_status ed_build_items(ed_sector s, int layout, int elem) {
+  if (items_ready(s, layout, elem)) return ED_OK;
+  ed_status ps = ED_OK;
+  cudaStream_t cs = ed_private_stream(&ps);
+  if (ps != ED_OK) return ps;
+  if (layout == 0) return build_list(s, layout, elem, cs);
+  // the orbital-factorised product reads no table of H_up: where the shape is
+  // known to take it, the ELL table waits until something else needs it
+  if (!(elem == 4 && fiber_group(s) && tuned_tiled(s, elem))) {
+    ED_TRY(ed_build_ell(s, cs));
+    ED_TRY(build_small_cols(s, cs));
+  }
+  ED_TRY(build_list(s, layout, elem, cs));
+  return decide_kernel(s, elem, cs);
 }
 
 // Slot of column c in a staged row group of ncp = 4 q4 columns: columns are
@@ -1633,33 +1645,42 @@ template ed_status ed_launch_hv<double>(ed_sector, const HvTables<double> &, int
                                         double *, int64_t *, cudaStream_t, double *const *, int,
                                         int64_t);
 
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy stream while another one captures
+  return true;
+}
+
 // Sector-order FP32 product through block-major order (see ed_takes_permuted).
-// *done = false: not taken (the rule, no memory for the scratch, or a stream
-// under capture, where the scratch would become part of the graph).
+// It needs the orbital-factorised product's lists and a scratch pair of
+// vectors, no ELL table and no timing.  *done = false: not taken, nothing
+// enqueued (the rule, no memory for lists or scratch, or a stream under
+// capture, where the scratch would become part of the graph); the
+// sector-order kernel, whose list is complete, then serves the call.
 static ed_status matvec_permuted(ed_sector s, const float *v, float *w, cudaStream_t st,
                                  bool *done) {
   *done = false;
   if (s->mp.norb < 2 || s->dim < ED_PERMUTE_MIN) return ED_OK;
   const int pinned = s->hv_pinned[0] ? s->hv_kernel[0] : -1;
-  if (!ed_takes_permuted(s->mp.norb, fiber_group(s), s->dim, pinned)) return ED_OK;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
+  if (!ed_takes_permuted(s->mp.norb, fiber_group(s), s->dim, pinned) || capturing(st))
     return ED_OK;
-  }
-  // both layouts' work lists, so that a later call under capture builds nothing
+  // the sector-order list too, so that a later call under capture builds nothing
   ED_TRY(ed_build_items(s, 0, 4));
-  ED_TRY(ed_build_items(s, 1, 4));
-  HvTables<float> tb = ed_hv_tables<float>(s, 1);
-  tb.small_cols = nullptr;  // the factorised product, whatever the tuner chose
   void *mem = nullptr;
-  if (ed_dmalloc(&mem, ed_permute_scratch(s->bdim), st, "permuted product") != ED_OK) {
+  ed_status rs = ED_OK;
+  cudaStream_t cs = ed_private_stream(&rs);
+  if (rs == ED_OK) rs = build_list(s, 1, 4, cs);
+  if (rs == ED_OK) rs = ed_dmalloc(&mem, ed_permute_scratch(s->bdim), st, "permuted product");
+  if (rs != ED_OK) {
     cudaGetLastError();
     ed_set_error_msg("");
     return ED_OK;
   }
+  HvTables<float> tb = ed_hv_tables<float>(s, 1);
+  tb.small_cols = nullptr;  // the factorised product, whatever the tuner chose
   float *bv = (float *)mem, *bw = bv + s->bdim;
-  ed_status rs = ed_permute_vec(s, ED_FP32, true, v, bv, st);
+  rs = ed_permute_vec(s, ED_FP32, true, v, bv, st);
   if (rs == ED_OK)
     rs = ed_launch_hv<float>(s, tb, HV_PLAIN, bv, bw, nullptr, nullptr, nullptr, nullptr, nullptr, st);
   if (rs == ED_OK) rs = ed_permute_vec(s, ED_FP32, false, bw, w, st);

@@ -60,3 +60,37 @@ def test_product_after_a_failed_allocation(ed, case, prec):
         return failed
 
     assert _failures(ed, call) >= 2
+
+
+def test_sector_order_product_needs_only_its_own_list(ed):
+    """A sector-order FP32 product that goes through block-major order (Norb=2 Ns=16) does
+    without it where an allocation of that way fails: only the sector-order list itself,
+    the first allocation, is needed.  Against the product with all memory there, both ways
+    within FP32 rounding (2 eps per term of rows of at most 32 terms of size below 10 |v|
+    with |v| <= 1/2)."""
+    m = make_model(2, 7, U=3.0, Jh=0.5, seed=12)
+    s = ed.Sector(m, 6, 6)
+    v = _vec(s.dim, torch.float32)
+    want = torch.empty_like(v)
+    ed.matvec(s, v, want, "fp32")
+    s.free()
+    tol = 2 * 2.0 ** -24 * 32 * 5.0
+
+    def call(n):
+        s = ed.Sector(m, 6, 6)
+        before = ed.kernel_launches()
+        ed.inject_alloc_failure(n)
+        w = torch.empty_like(v)
+        if n == 1:
+            with pytest.raises(ed.EDError) as e:
+                ed.matvec(s, v, w, "fp32")
+            assert e.value.status == ed.ED_ERR_OOM
+        else:
+            ed.matvec(s, v, w, "fp32")
+            launches = ed.kernel_launches() - before
+            assert float((w - want).abs().max()) <= tol
+        ed.inject_alloc_failure(0)
+        s.free()
+        return n == 1 or launches == 1  # one launch: the sector-order kernel
+
+    assert _failures(ed, call) >= 4

@@ -15,8 +15,9 @@ def _vec(n, dt, seed=1):
 
 
 def test_sector_order_product_below_the_crossover_stays_in_its_layout(ed):
-    """Norb=2 Ns=14 (7,7): the sector-order kernel, one launch; with the
-    tiled family pinned, through block-major order."""
+    """Norb=2 Ns=14 (7,7): the sector-order kernel, one launch (no
+    block-major lists, nothing timed); with the tiled family pinned, through block-major
+    order."""
     s = ed.Sector(make_model(2, 6, U=3.0, Jh=0.5, seed=12), 7, 7)
     v = _vec(s.dim, torch.float32)
     w = torch.empty_like(v)
@@ -27,4 +28,18 @@ def test_sector_order_product_below_the_crossover_stays_in_its_layout(ed):
     before = ed.kernel_launches()
     ed.matvec(s, v, w, "fp32")
     assert ed.kernel_launches() - before >= 4
+    s.free()
+
+
+def test_first_call_through_block_major_order_times_nothing(ed):
+    """Norb=2 Ns=16 (6,6): both permutations, the H_up pass (one launch: no block is
+    wider than 4912 columns) and the H_dw pass, also on the shape's first call: no ELL
+    table is built and no kernel is timed for it."""
+    s = ed.Sector(make_model(2, 7, U=3.0, Jh=0.5, seed=12), 6, 6)
+    v = _vec(s.dim, torch.float32)
+    w = torch.empty_like(v)
+    for _ in range(2):
+        before = ed.kernel_launches()
+        ed.matvec(s, v, w, "fp32")
+        assert ed.kernel_launches() - before == 4
     s.free()
