@@ -146,8 +146,8 @@ ed_status ed_sector_free(ed_sector s);
  * Large FP32 sectors of several orbitals go through block-major order where
  * that is the faster way (from 2^25 elements with two or three orbitals, 2^27
  * with four; from 2^20 where ed_sector_set_kernel pinned the tiled family),
- * in a scratch of two vectors that returns to the library's pool
- * (ed_memory_trim).  Without memory for it, and on a stream under
+ * in a scratch of two vectors, at most 2 GiB, that returns to the library's
+ * pool (ed_memory_trim).  Without memory for it, and on a stream under
  * capture, the sector-order kernel serves the call: the same sum of the same
  * terms in another order, so w can differ in its last bits between two such
  * calls (about 1e-7 of sum_k |H_ik v_k|). */

@@ -37,11 +37,15 @@ constexpr bool ed_takes_rows(int elem, int64_t ddw, int64_t stride) {
 // group: levels of an orbital group, 0 where the factorised product does not
 // apply; pinned: the kernel the caller chose for the block-major layout (0 the
 // tiled family, which is then taken from 2^20 elements on, 1 element-parallel,
-// -1 none).
+// -1 none).  The scratch stays cached in the library's pool, so it is bounded:
+// above ED_PERMUTE_SCRATCH_MAX the sector-order kernel runs.
 constexpr int64_t ED_PERMUTE_MIN = (int64_t)1 << 20;
+constexpr int64_t ED_PERMUTE_SCRATCH_MAX = (int64_t)2 << 30;
 constexpr int64_t ed_permute_scratch(int64_t bdim) { return 2 * bdim * (int64_t)sizeof(float); }
-constexpr bool ed_takes_permuted(int norb, int group, int64_t dim, int pinned) {
-  if (group == 0 || dim < ED_PERMUTE_MIN || pinned == 1) return false;
+constexpr bool ed_takes_permuted(int norb, int group, int64_t dim, int64_t bdim, int pinned) {
+  if (group == 0 || dim < ED_PERMUTE_MIN || pinned == 1 ||
+      ed_permute_scratch(bdim) > ED_PERMUTE_SCRATCH_MAX)
+    return false;
   if (pinned == 0) return true;
   return norb <= 3 ? dim >= (int64_t)1 << 25 : norb == 4 && dim >= (int64_t)1 << 27;
 }

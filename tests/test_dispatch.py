@@ -47,7 +47,8 @@ def test_rows_kernel_within_its_32_bit_units(tmp_path):
 
 def test_sector_order_detour_rule(tmp_path):
     """The sector-order FP32 product goes through block-major order only where that was
-    measured faster, and follows a pinned kernel."""
+    measured faster, never with a scratch above 2 GiB, and follows a pinned kernel."""
+    G = 1 << 30
     cases = [  # norb, group, dim, bdim, pinned, want
         (2, 7, 11778624, 11806080, -1, 0),      # Norb=2 Ns=14 (7,7): slower
         (2, 8, 165636900, 165791340, -1, 1),    # Norb=2 Ns=16 (8,8)
@@ -56,11 +57,14 @@ def test_sector_order_detour_rule(tmp_path):
         (4, 4, 165636900, 166000000, -1, 1), (4, 4, 102951200, 103200000, -1, 0),
         (5, 3, 41409225, 41900000, -1, 0),      # five orbitals: never faster
         (2, 0, 2363904400, 2364000000, -1, 0),  # groups the factorised product does not take
+        (3, 6, 2363904400, 2364487840, -1, 0),  # Norb=3 Ns=18: 19 GB of scratch
+        (3, 6, 2363904400, 2364487840, 0, 0),
+        (2, 8, G // 4, G // 4, -1, 1), (2, 8, G // 4, G // 4 + 1, -1, 0),
         (2, 8, 1 << 25, 1 << 25, -1, 1), (2, 8, (1 << 25) - 1, 1 << 25, -1, 0),
         (4, 4, 1 << 27, 1 << 27, -1, 1), (4, 4, (1 << 27) - 1, 1 << 27, -1, 0),
         (2, 7, 6012006, 6030000, 0, 1), (2, 7, (1 << 20) - 1, 1 << 20, 0, 0),  # tiled pinned
         (5, 3, 1 << 20, 1 << 20, 0, 1), (2, 8, 165636900, 165791340, 1, 0),    # pinned
     ]
-    got = _run(tmp_path, "\n".join('printf("%%d\\n", (int)ed_takes_permuted(%d, %d, %dLL, %d));'
-                                   % (c[0], c[1], c[2], c[4]) for c in cases))
+    got = _run(tmp_path, "\n".join('printf("%%d\\n", (int)ed_takes_permuted(%d, %d, %dLL, %dLL, %d));'
+                                   % c[:5] for c in cases))
     assert got == [c[5] for c in cases]
