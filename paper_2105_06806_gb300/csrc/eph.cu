@@ -241,8 +241,8 @@ extern "C" ed_status ed_eph_matvec(ed_sector s, const ed_phonon *ph, ed_precisio
     return ED_ERR_ARG;
   }
   cudaStream_t cs = (cudaStream_t)stream;
-  // sector-order slices that are block-major as they are (see matvec_layout)
-  const int layout = ed_same_layout(s) && (((uintptr_t)d_v | (uintptr_t)d_w) & 15) == 0 ? 1 : 0;
+  int layout = 0;
+  ED_TRY(ed_sector_order_layout(s, prec == ED_FP64 ? 8 : 4, d_v, d_w, cs, &layout));
   if (prec == ED_FP64) {
     ED_TRY(ed_build_items(s, layout, 8));
     return eph_apply<double>(s, pp, layout, (const double *)d_v, (double *)d_w, cs);

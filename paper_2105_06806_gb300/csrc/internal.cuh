@@ -453,6 +453,14 @@ ed_status ed_launch_hv(ed_sector s, const HvTables<T> &tb, int mode, const T *v,
 // True when vectors in sector order are block-major vectors as they are: one
 // orbital (the two orders agree) with no padding columns.
 inline bool ed_same_layout(ed_sector s) { return s->mp.norb == 1 && s->bstride == s->sp[0].dim; }
+// The layout a call on sector-order vectors runs in.  1: the vectors are
+// block-major as they are and 16-byte aligned, so they take that layout's
+// kernels (ELL table and 16-byte accesses instead of CSR rows; the same w bit
+// for bit), whose tables the first such call builds.  Where that fails (no
+// memory for the tables or the autotuner's vectors) or the stream is under
+// capture, 0: the sector-order kernel needs its own list alone.
+ed_status ed_sector_order_layout(ed_sector s, int elem, const void *v, const void *w,
+                                 cudaStream_t st, int *layout);
 
 int64_t ed_hv_num_parts(ed_sector s, int layout, int elem_size);
 template <typename T>

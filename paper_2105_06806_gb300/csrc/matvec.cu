@@ -1689,6 +1689,24 @@ static ed_status matvec_permuted(ed_sector s, const float *v, float *w, cudaStre
   return rs;
 }
 
+ed_status ed_sector_order_layout(ed_sector s, int elem, const void *v, const void *w,
+                                 cudaStream_t st, int *layout) {
+  *layout = 0;
+  if (!ed_same_layout(s) || (((uintptr_t)v | (uintptr_t)w) & 15)) return ED_OK;
+  // the sector-order list too, so that a later call under capture builds nothing
+  ED_TRY(ed_build_items(s, 0, elem));
+  if (!items_ready(s, 1, elem)) {
+    if (capturing(st)) return ED_OK;
+    if (ed_build_items(s, 1, elem) != ED_OK) {
+      cudaGetLastError();
+      ed_set_error_msg("");
+      return ED_OK;
+    }
+  }
+  *layout = 1;
+  return ED_OK;
+}
+
 static ed_status matvec_layout(ed_sector s, ed_precision prec, const void *d_v, void *d_w,
                                int64_t n, void *stream, int layout) {
   if (!s || !d_v || !d_w || d_v == d_w) return ED_ERR_ARG;
@@ -1704,10 +1722,8 @@ static ed_status matvec_layout(ed_sector s, ed_precision prec, const void *d_v, 
                                  : "vectors must be aligned to their element size");
     return ED_ERR_ARG;
   }
-  // sector-order vectors that are block-major as they are take that layout's
-  // kernels (ELL table and 16-byte accesses instead of CSR rows)
-  if (layout == 0 && ed_same_layout(s) && (((uintptr_t)d_v | (uintptr_t)d_w) & 15) == 0) layout = 1;
   cudaStream_t st = (cudaStream_t)stream;
+  if (layout == 0) ED_TRY(ed_sector_order_layout(s, prec == ED_FP64 ? 8 : 4, d_v, d_w, st, &layout));
   if (prec == ED_FP64) {
     ED_TRY(ed_build_items(s, layout, 8));
     return ed_launch_hv<double>(s, ed_hv_tables<double>(s, layout), HV_PLAIN,

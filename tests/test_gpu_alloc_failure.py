@@ -94,3 +94,72 @@ def test_sector_order_product_needs_only_its_own_list(ed):
         return n == 1 or launches == 1  # one launch: the sector-order kernel
 
     assert _failures(ed, call) >= 4
+
+
+@pytest.mark.parametrize("nph", [None, 3])
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_one_orbital_product_needs_only_its_own_list(ed, prec, nph):
+    """Sector-order vectors of one orbital that are block-major as they are (D_up = 924)
+    take that layout's kernels; where an allocation for those fails the call runs on the
+    sector-order list, its first allocation: the same w bit for bit.  nph: the coupled
+    product."""
+    m = make_model(1, 11, U=2.0, seed=4)
+    ph = ed.phonon(0.5, [0.3], nph or 0)
+
+    def product(s, v, w):
+        if nph is None:
+            ed.matvec(s, v, w, prec)
+        else:
+            ed.eph_matvec(s, ph, v, w, prec)
+
+    s = ed.Sector(m, 6, 5)
+    v = _vec(s.dim * ((nph or 0) + 1), DT[prec])
+    want = torch.empty_like(v)
+    product(s, v, want)
+    # both lists exist now: vectors at an odd element allocate nothing
+    off = [torch.empty(v.numel() + 1, device="cuda", dtype=DT[prec])[1:] for _ in range(2)]
+    off[0].copy_(v)
+    ed.inject_alloc_failure(1)
+    product(s, off[0], off[1])
+    ed.inject_alloc_failure(0)
+    assert torch.equal(off[1], want)
+    s.free()
+
+    def call(n):
+        s = ed.Sector(m, 6, 5)
+        ed.inject_alloc_failure(n)
+        w = torch.empty_like(v)
+        if n == 1:
+            with pytest.raises(ed.EDError) as e:
+                product(s, v, w)
+            assert e.value.status == ed.ED_ERR_OOM
+        else:
+            product(s, v, w)
+            assert torch.equal(w, want)
+        ed.inject_alloc_failure(0)
+        s.free()
+
+    for n in range(1, 10):
+        call(n)
+
+
+def test_one_orbital_product_under_capture(ed):
+    """Captured before the block-major tables exist (an earlier call on vectors at an odd
+    element built the sector-order list): nothing is built under capture, and the replayed
+    product is the same w bit for bit."""
+    s = ed.Sector(make_model(1, 11, U=2.0, seed=4), 6, 5)
+    x = _vec(s.dim + 1, torch.float32)
+    v, w = x[:-1], torch.empty(s.dim, device="cuda")
+    off = torch.empty(s.dim + 1, device="cuda")[1:]
+    y = torch.empty(s.dim + 1, device="cuda")[1:]
+    off.copy_(v)
+    ed.matvec(s, off, y, "fp32")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        ed.inject_alloc_failure(1)
+        ed.matvec(s, v, w, "fp32")
+        ed.inject_alloc_failure(0)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(w, y)
+    s.free()
