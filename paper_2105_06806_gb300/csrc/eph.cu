@@ -145,10 +145,12 @@ ed_status eph_apply(ed_sector s, const PhParams &ph, int layout, const T *v, T *
                     cudaStream_t cs, const HvTables<T> *tables = nullptr) {
   HvTables<T> tb = tables ? *tables : ed_hv_tables<T>(s, layout);
   const int64_t slice = layout == 1 ? s->bdim : s->dim;
-  // the sector's kernel was chosen on one slice: with all slices in a launch
-  // the FP32 tiled family has the work to fill the GPU and is the faster one
-  // (the same w bit for bit)
-  if (sizeof(T) == 4 && slice * (ph.nph + 1) >= (int64_t)1 << 22) tb.small_cols = nullptr;
+  // the tuner chose the sector's kernel on one slice: with several slices in a
+  // launch the FP32 tiled family has the work to fill the GPU and is the faster
+  // one (the same w bit for bit)
+  if (sizeof(T) == 4 && !s->hv_pinned[0] && ph.nph > 0 &&
+      slice * (ph.nph + 1) >= (int64_t)1 << 22)
+    tb.small_cols = nullptr;
   // every slice in one launch: a slice of a small sector does not fill the GPU.
   // Bound: the product's shared-memory gathers (62 us), then k_phonon on
   // L2-resident slices (15 us, 7.4 TB/s).  Norb=1 Ns=12, 11 slices, FP32: 85 us
