@@ -471,8 +471,9 @@ ed_status launch_one(const HvLaunch<float> *a, int mode, unsigned ns, cudaStream
   if constexpr ((fiber_shapes(G) >> SHAPE) & 1) {
     constexpr int smem = 2 * Shape<G, SHAPE>::CAP * (int)sizeof(float);
     if (!a) {  // opt into large shared memory
-      ED_TRY_CUDA(cudaFuncSetAttribute(k_hv_fiber<G, SHAPE>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      if ((mode >> SHAPE) & 1)
+        ED_TRY_CUDA(cudaFuncSetAttribute(k_hv_fiber<G, SHAPE>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     } else if (n > 0) {
       k_hv_fiber<G, SHAPE><<<dim3((unsigned)n, ns), Shape<G, SHAPE>::NT, smem, st>>>(
           *a, mode == HV_LANCZOS);
@@ -484,7 +485,9 @@ ed_status launch_one(const HvLaunch<float> *a, int mode, unsigned ns, cudaStream
 }
 
 // One launch per shape that the sector's items need; a == nullptr: prepares
-// the kernels of this G on the current device.
+// the kernels of this G and the shapes in `mode` (bit per shape) on the current
+// device.  Only those a sector has items for: an instance is a megabyte of
+// code and more, which the driver loads on first use: all of them 11 ms.
 template <int G>
 ed_status launch_g(const HvLaunch<float> *a, int mode, unsigned ns, cudaStream_t st) {
   if (a && mode != HV_PLAIN && mode != HV_LANCZOS) return ED_ERR_ARG;

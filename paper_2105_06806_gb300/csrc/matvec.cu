@@ -150,7 +150,8 @@ constexpr int DW_COLS = 512;   // columns of an item (a multiple of 4)
 static bool passa_is_wide(ed_sector s);
 static int64_t widest_block(ed_sector s);  // padded columns of the widest up block
 
-// fiber.cuh: launch of the orbital-factorised product (a = nullptr: prepare)
+// fiber.cuh: launch of the orbital-factorised product (a = nullptr: prepares
+// the CTA shapes in `mode`)
 namespace fiber {
 template <int G>
 ed_status launch_g(const HvLaunch<float> *a, int mode, unsigned ns, cudaStream_t st);
@@ -740,6 +741,11 @@ static ed_status build_list(ed_sector s, int layout, int elem, cudaStream_t cs) 
         items.push_back(HvItem{(int32_t)r, (int32_t)std::min<int64_t>(R, R1 - r), (int32_t)C0,
                                (int32_t)nc, (int32_t)op_up[bu], deg, eoff, ncp});
     }
+  }
+  if (fiber) {
+    int shapes = 0;
+    for (int k = 0; k < FIBER_SHAPES; ++k) shapes |= (nfib[k] > 0) << k;
+    ED_TRY(launch_fiber(fiber, nullptr, shapes, 1, nullptr));
   }
   ItemList t;
   t.nitems = (int64_t)items.size();
@@ -1543,8 +1549,6 @@ ed_status ed_hv_prepare() {
   if (dev < 64 && done[dev]) return ED_OK;
   ED_TRY((prepare_layout<T, false>()));
   ED_TRY((prepare_layout<T, true>()));
-  if (sizeof(T) == 4)
-    for (int g = FIBER_MIN_G; g <= FIBER_MAX_G; ++g) ED_TRY(launch_fiber(g, nullptr, 0, 1, nullptr));
   if (dev < 64) done[dev] = true;
   return ED_OK;
 }
