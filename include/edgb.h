@@ -201,11 +201,12 @@ ed_status ed_sector_blocked_kernel(ed_sector s, ed_precision prec, int32_t *kern
 
 /* Autotuner (no counterpart in the paper).  Sectors of at most 2^17 padded
  * elements use the element-parallel kernel; above that the first sector of
- * each model shape (Norb, Nbath, precision) times the tiled family and
+ * each model shape (Norb, Nbath, precision) and, in FP32, of each factor of 8
+ * in padded elements (2^17, 2^20, 2^23, ..) times the tiled family and
  * the element-parallel kernel (one warm-up and three launches each, on two
  * scratch vectors of the sector's size) when its block-major tables are
- * built, and every sector of that shape in the process then uses the faster
- * one.
+ * built, and every sector of that shape and size in the process then uses the
+ * faster one.
  * ed_sector_tune_info returns the kernel in use and host_ms[0..1], the
  * measured milliseconds of the tiled and the element-parallel product
  * (-1 where this sector did not time them).  ed_sector_set_kernel pins a

@@ -93,16 +93,13 @@ __device__ __forceinline__ void vec_get(const float2 &v, float *x) {
 }
 
 // Element-parallel product (one thread per element of the padded block-major
-// vector, striding for large sectors).  Below EDGB_TUNE_MIN elements the
+// vector, striding for large sectors).  Below ED_TUNE_MIN elements the
 // tiled kernel has too few work items to fill the GPU and its time is set by
 // the serial per-thread tile, so the element-parallel kernel is used; above
 // it, which one is faster depends on the block shapes and the precision (the
 // tiled kernel reuses staged rows and ELL entries, the element-parallel one
 // keeps more loads in flight): the autotuner times both.
 constexpr int HVS_THREADS = 256;
-#ifndef EDGB_TUNE_MIN
-#define EDGB_TUNE_MIN (1 << 17)
-#endif
 // Elements per thread of the element-parallel product: 1 up to
 // EDGB_SMALL_PARTS CTAs, then K, so that the grid (= the Lanczos partials)
 // stays within EDGB_SMALL_PARTS.  CTA b takes the K consecutive 256-element
@@ -523,26 +520,24 @@ static ed_status build_dw_items(ed_sector s, ItemList &il, int elem, cudaStream_
 
 // ----------------------------------------------------------------- autotuner
 //
-// For sectors above EDGB_TUNE_MIN padded elements the faster of the tiled
+// For sectors above ED_TUNE_MIN padded elements the faster of the tiled
 // family (one or two passes) and the element-parallel product depends on the
 // block shapes and the precision, so it is measured: both kernels, one
 // warm-up and three timed launches each (alternating) on a scratch vector,
-// on this thread's private stream.  The choice is kept per model shape
-// (Norb, Nbath, precision) for the life of the process, so every sector of a
-// shape uses the same kernel and results do not depend on which call came
-// first.  The sectors of one shape share the block structure that decides
-// between the kernels (block widths set by the orbital count, bath strings
-// of one length); where two sectors of a shape were measured (Ns = 14, at
-// and next to half filling) both chose the same kernel wherever the two
-// kernels differed by more than 5%.  Keying on the sector as well made
-// a serving stream whose requests are mostly distinct sectors tune on almost
-// every request (15% fewer solves/s at Ns <= 16).  Both kernels give the
-// same w = H v bit for bit.
+// on this thread's private stream.  The choice is kept per model shape,
+// precision and size class (ed_tune_class) for the life of the process, so
+// every such sector uses the same kernel.  The sectors of one shape share the
+// block structure (block widths set by the orbital count, bath strings of one
+// length).  Keying on the sector as well made a serving stream whose requests
+// are mostly distinct sectors tune on almost every request (15% fewer solves/s
+// at Ns <= 16).  Both kernels give the same w = H v bit for bit.
 namespace {
 struct TuneKey {
-  int norb, nbath, elem;
+  int norb, nbath, elem, size;
+  TuneKey(ed_sector s, int elem)
+      : norb(s->mp.norb), nbath(s->mp.nbath), elem(elem), size(ed_tune_class(elem, s->bdim)) {}
   bool operator<(const TuneKey &o) const {
-    return std::tie(norb, nbath, elem) < std::tie(o.norb, o.nbath, o.elem);
+    return std::tie(norb, nbath, elem, size) < std::tie(o.norb, o.nbath, o.elem, o.size);
   }
 };
 std::mutex g_tune_mu;
@@ -571,9 +566,9 @@ __global__ void k_tune_fill(T *v, int64_t n, int64_t stride, const int32_t *padi
 static bool tuned_tiled(ed_sector s, int elem) {
   const int8_t k = s->hv_kernel[elem == 8 ? 1 : 0];
   if (k >= 0) return k == 0;
-  if (s->bdim <= (int64_t)EDGB_TUNE_MIN) return false;
+  if (s->bdim <= ED_TUNE_MIN) return false;
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  const auto it = g_tune.find(TuneKey{s->mp.norb, s->mp.nbath, elem});
+  const auto it = g_tune.find(TuneKey(s, elem));
   return it != g_tune.end() && it->second == 0;
 }
 
@@ -625,11 +620,11 @@ static ed_status decide_kernel(ed_sector s, int elem, cudaStream_t cs) {
     s->hv_kernel[e] = 0;
     return ED_OK;
   }
-  if (s->bdim <= (int64_t)EDGB_TUNE_MIN) {
+  if (s->bdim <= ED_TUNE_MIN) {
     s->hv_kernel[e] = 1;
     return ED_OK;
   }
-  const TuneKey key{s->mp.norb, s->mp.nbath, elem};
+  const TuneKey key(s, elem);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(key);
