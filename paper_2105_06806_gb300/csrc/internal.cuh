@@ -423,6 +423,8 @@ struct LanczosState {
   int32_t maxit;
   int32_t check_every;  // fewest steps between two Ritz-value tests
   int32_t next_check;   // step of the next scheduled test
+  int32_t last_check;   // step of the last test
+  int32_t ran;          // steps run (above j where an earlier step ended the run)
   int32_t pad_;
   double check_growth;  // a test at step k schedules the next one
                         // max(check_every, ceil(check_growth * k)) steps later

@@ -122,6 +122,32 @@ __device__ int sturm_count(const double *a, const double *b2, int k, double x) {
   return cnt;
 }
 
+// Largest q <= k for which T_q has fewer than two eigenvalues below x: the
+// leading principal minors of one recurrence give the counts of all q.
+__device__ int last_single(const double *a, const double *b2, int k, double x) {
+  double pm = 1.0, p = a[0] - x;
+  int cnt = 0;
+  if (p <= 0.0) {
+    if (p == 0.0) p = -1e-300;
+    cnt = 1;
+  }
+  for (int i = 1; i < k; ++i) {
+    double pn = (a[i] - x) * p - b2[i] * pm;
+    if (is_zero(pn)) pn = neg_bit(p) ? 1e-300 : -1e-300;
+    cnt += neg_bit(pn) != neg_bit(p);
+    if (cnt >= 2) return i;
+    pm = p;
+    p = pn;
+    const int e = bexp(p);
+    if (out_of_range(e)) {
+      const double f = rescale_factor(e);
+      p *= f;
+      pm *= f;
+    }
+  }
+  return k;
+}
+
 // Squared last component of the normalised eigenvector of T_k for the
 // eigenvalue theta: -p_{k-1}(theta) / p_k'(theta).
 __device__ double last_component_sq(const double *a, const double *b2, int k, double x) {
@@ -380,14 +406,17 @@ __global__ void __launch_bounds__(AXPY_THREADS) k_axpy_norm(LanczosState *st, T 
 }
 
 // beta_{j+1}, scale, Ritz value and stop test.  The Ritz value is evaluated
-// at steps 1 and 2, at the scheduled steps (next_check) and at the last step.
+// at steps 1 and 2, at the scheduled steps (next_check) and at the last step; a
+// test that finds a copy of a converged state also looks at steps since the
+// last test, and a run then ends on the earlier step (j below the steps run).
 __global__ void k_beta(LanczosState *st, const double *part, int64_t nparts) {
   __shared__ double red[SCALAR_THREADS / 32];
   __shared__ int stop;
   // T_k, its squared off-diagonal, then (inverse iteration) pivots and y
   __shared__ double s_a[ED_MAX_LANCZOS], s_b[ED_MAX_LANCZOS], s_b2[ED_MAX_LANCZOS];
   __shared__ double s_rp[ED_MAX_LANCZOS], s_y[ED_MAX_LANCZOS];
-  __shared__ double s_be, s_hint[2];
+  __shared__ double s_be, s_hint[2], s_rest, s_restq;
+  __shared__ int copies, s_cand[4];
   if (st->done) return;
   double s2 = cta_sum_parts(part, nparts, red);
   const double c2 = cta_sum_parts(part + nparts, nparts, red);  // <w, v_j>
@@ -407,6 +436,7 @@ __global__ void k_beta(LanczosState *st, const double *part, int64_t nparts) {
   }
   __syncthreads();
   const int k = j + 1;
+  int kc = k;  // the step the run ends on, where it converges
   const bool scheduled = k >= st->next_check;
   const bool want = st->tol > 0.0 && (stop != 0 || scheduled || k <= 2);
   if (want) {
@@ -419,37 +449,86 @@ __global__ void k_beta(LanczosState *st, const double *part, int64_t nparts) {
                                              : -1e300;
     }
     __syncthreads();
-    const double th = lowest_eigenvalue(s_a, s_b, s_b2, k, s_hint[0], s_hint[1]);
-    __shared__ int ritz;
-    if (threadIdx.x == 0) {
-      const double be = s_be;
-      double y2 = last_component_sq(s_a, s_b2, k, th);
-      double rest = be * sqrt(y2);
-      // The polynomial formula loses relative accuracy once the Ritz value
-      // has converged; near convergence use inverse iteration instead.
-      ritz = rest < 1e-6 * fmax(1.0, fabs(th));
-      if (ritz) {
+    double th = lowest_eigenvalue(s_a, s_b, s_b2, k, s_hint[0], s_hint[1]);
+    // a second Ritz value near theta (counted by another warp meanwhile): from
+    // about 3e-8 on the three sweeps below leave enough of it in the vector to
+    // hide a residual of 1e-13
+    if (threadIdx.x == 32)
+      copies = k > 2 && sturm_count(s_a, s_b2, k, th + 1e-6 * fmax(1.0, fabs(th))) >= 2;
+    if (threadIdx.x == 0) s_rest = s_be * sqrt(last_component_sq(s_a, s_b2, k, th));
+    __syncthreads();
+    // The polynomial formula loses relative accuracy once the Ritz value
+    // has converged; near convergence use inverse iteration instead.
+    double rest = s_rest;
+    bool ritz = rest < 1e-6 * fmax(1.0, fabs(th));  // s_y holds the Ritz vector
+    if (ritz) {
+      __syncthreads();
+      if (threadIdx.x == 0) {
         // the last component is tiny near convergence: three sweeps push the
         // other eigencomponents well below it
         ritz_vector(s_a, s_b, k, th, 3, s_rp, s_b2, s_y);
-        rest = be * fabs(s_y[k - 1]);
+        s_rest = s_be * fabs(s_y[k - 1]);
       }
+      __syncthreads();
+      rest = s_rest;
+    }
+    // converged, also when the test falls on the max_iter step
+    bool conv = (stop == 0 || stop == 3) && k >= 2 && rest <= st->tol * fmax(1.0, fabs(th));
+    // Rounding lets copies of a converged state appear.  While a copy comes near
+    // theta the Ritz vector mixes with it and the estimate is large again: the
+    // steps that met the tolerance lie between two tests.  The last step whose
+    // second Ritz value was still clearly above theta (four distances, from 1e-4
+    // down to 1e-10, so that one of them is below the spacing of the spectrum) is
+    // one of them; it is tested as if the schedule had named it.
+    if (!conv && copies && stop != 2) {
+      for (int i = threadIdx.x; i < k; i += blockDim.x) s_b2[i] = s_b[i] * s_b[i];
+      __syncthreads();
+      if (threadIdx.x < 4) {
+        double d = 1e-4;
+        for (int t = 0; t < (int)threadIdx.x; ++t) d *= 1e-2;
+        s_cand[threadIdx.x] = last_single(s_a, s_b2, k, th + d * fmax(1.0, fabs(th)));
+      }
+      __syncthreads();
+      for (int t = 0; t < 4 && !conv; ++t) {
+        const int q = s_cand[t];
+        if (q < 2 || q <= st->last_check || q >= k || (t > 0 && q == s_cand[t - 1])) continue;
+        for (int i = threadIdx.x; i < k; i += blockDim.x) s_b2[i] = s_b[i] * s_b[i];
+        __syncthreads();
+        const double tq = lowest_eigenvalue(s_a, s_b, s_b2, q, 1e300, -1e300);
+        if (threadIdx.x == 0) {
+          ritz_vector(s_a, s_b, q, tq, 3, s_rp, s_b2, s_y);
+          s_restq = s_b[q] * fabs(s_y[q - 1]);
+        }
+        ritz = false;  // s_y is no longer the vector of T_k
+        __syncthreads();
+        if (s_restq <= st->tol * fmax(1.0, fabs(tq))) {
+          conv = ritz = true;
+          th = tq;
+          rest = s_restq;
+          kc = q;
+        }
+        __syncthreads();
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
       st->acc[3] = isfinite(prev) ? th - prev : 1e300;
       st->theta = th;
       st->rest = rest;
-      // converged, also when the test falls on the max_iter step
-      if ((stop == 0 || stop == 3) && rest <= st->tol * fmax(1.0, fabs(th)) && k >= 2) stop = 1;
+      st->last_check = k;
+      if (conv) stop = 1;
       if (scheduled)
         st->next_check = k + max(st->check_every, (int)ceil(st->check_growth * (double)k));
     }
     __syncthreads();
     if (ritz)
-      for (int i = threadIdx.x; i < k; i += blockDim.x) st->y[i] = s_y[i];
+      for (int i = threadIdx.x; i < kc; i += blockDim.x) st->y[i] = s_y[i];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     if (stop) st->done = stop;
-    st->j = k;
+    st->j = kc;
+    st->ran = k;
   }
 }
 
@@ -530,6 +609,8 @@ __global__ void k_state_init(LanczosState *st, const double *part, int64_t npart
     st->maxit = maxit;
     st->check_every = check_every;
     st->next_check = check_every;
+    st->last_check = 0;
+    st->ran = 0;
     st->check_growth = check_growth;
     st->tol = tol;
     st->tnorm = 0.0;
@@ -1137,7 +1218,7 @@ static ed_status lanczos_solve(ed_sector s, int maxit, double tol, uint64_t seed
   ED_TRY_CUDA(cudaMemcpyAsync(h_state, st, sizeof(LanczosState), cudaMemcpyDeviceToHost, cs));
   ED_TRY_CUDA(cudaStreamSynchronize(cs));
   const int k = h_state->j;
-  int mv = k;
+  int mv = h_state->ran;
   if (want_vector && k > 0) {
     k_tridiag_vector<<<1, TRIDIAG_THREADS, 5 * sizeof(double) * ED_MAX_LANCZOS, cs>>>(st, k);
     ED_LAUNCHED(1);
