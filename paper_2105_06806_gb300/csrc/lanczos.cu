@@ -68,13 +68,6 @@ template <>
 __device__ __forceinline__ double fmaT<double>(double a, double b, double c) {
   return __fma_rn(a, b, c);
 }
-template <typename T>
-__device__ __forceinline__ T mulT(T a, T b);
-template <>
-__device__ __forceinline__ float mulT<float>(float a, float b) { return __fmul_rn(a, b); }
-template <>
-__device__ __forceinline__ double mulT<double>(double a, double b) { return __dmul_rn(a, b); }
-
 // ----------------------------------------------------------------- tridiagonal
 
 // The helpers below read T_k from shared-memory copies: a[i] = alpha_i,
@@ -1082,7 +1075,7 @@ static ed_status second_pass(ed_sector s, const HvTables<T> &tb, T *const *bufs,
   // then the streaming update, which here also adds y_j v_j into psi) instead
   // of the fused second-pass H_dw epilogue: 14.3 + 3 ms against 19.6 ms per
   // step at Ns=18; the same operations, so the same vectors bit for bit.
-  const bool split = (tb.ditems || tb.fiber) && !tb.small_cols;
+  const bool split = tb.ditems && !tb.small_cols;
   for (int j = j0; j + 1 < k; ++j) {
     if (split) {
       int64_t np1 = 0;

@@ -1168,13 +1168,14 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : EDGB_MIN_CTAS) k_hv(HvLau
 }
 
 // Second pass of the two-pass product: out += H_dw v over DwItems (rows of
-// one dw block x a column chunk of one up block), then the epilogue of k_hv.
+// one dw block x a column chunk of one up block), then the epilogue of k_hv
+// (plain, sliced or Lanczos mode: the second pass of a ground state runs the
+// Lanczos mode and the update kernel on these sectors).
 // Items run column chunk by column chunk through all rows of a dw block, so
 // the chunk's strip of v (rows of the dw block x chunk columns) is the L2
 // working set of the neighbour-row reads.  Each accumulator continues from
 // the first pass's value and adds the H_dw terms in the same order as k_hv,
 // so the product equals the one-pass product bit for bit.
-
 //
 // A thread takes RT rows x 4 columns, NB neighbour rows in flight.  Blocks
 // narrower than an item leave most threads of a tall tile without work: there
@@ -1187,34 +1188,23 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
   __shared__ T s_dval[DW_ROWS * ED_MAX_NS];
   __shared__ int32_t s_dn[DW_ROWS];
   const HvTables<T> &tb = a.tb;
-  int j = 0;
-  T s_cur = T(1), s_prev = T(1), beta_s = T(0), alpha_s = T(0), y_s = T(0);
+  T s_cur = T(1);
   const T *g;
-  const T *prev = nullptr;
   T *out;
   if (ed_hv_plain(MODE)) {
     g = MODE == HV_SLICED ? a.v + blockIdx.y * a.slice : a.v;
     out = MODE == HV_SLICED ? a.w + blockIdx.y * a.slice : a.w;
   } else {
     const LanczosState *st = a.st;
-    if (MODE == HV_LANCZOS && st->done) return;
-    j = st->j;
-    const int m3 = j % 3;
+    if (st->done) return;
+    const int j = st->j, m3 = j % 3;
     g = m3 == 0 ? a.b0 : (m3 == 1 ? a.b1 : a.b2);
     out = m3 == 0 ? a.b1 : (m3 == 1 ? a.b2 : a.b0);
-    prev = m3 == 0 ? a.b2 : (m3 == 1 ? a.b0 : a.b1);
-    if (MODE == HV_LANCZOS && a.basis) {
+    if (a.basis) {
       g = a.basis[j];
-      prev = a.basis[j > 0 ? j - 1 : 0];
       out = a.basis[j + 1];
     }
     s_cur = (T)st->scale[m3];
-    if (MODE == HV_SECOND) {
-      s_prev = (T)st->scale[(j + 2) % 3];
-      beta_s = coef_of<T>(st->beta[j], st->scale[(j + 2) % 3]);
-      alpha_s = coef_of<T>(st->alpha[j], st->scale[m3]);
-      y_s = (T)(st->y[j] * st->scale[m3]);
-    }
   }
   const DwItem it = tb.ditems[blockIdx.x];
   const int64_t stride = tb.stride;
@@ -1278,17 +1268,9 @@ __global__ void __launch_bounds__(DW_THREADS) k_hv_dw(HvLaunch<T> a) {
         if (ed_hv_plain(MODE)) {
           out[gi] = acc[i][u];
         } else {
-          const T x = g[gi];
-          T w1 = mul_t<T>(acc[i][u], s_cur);
-          if (MODE == HV_SECOND && j > 0)  // the Lanczos step does this in its update
-            w1 = fma_t<T>(-beta_s, vec_of<T>(prev[gi], s_prev), w1);
-          if (MODE == HV_LANCZOS) {
-            out[gi] = w1;
-            dot = fma_t<T>(vec_of<T>(x, s_cur), w1, dot);
-          } else {
-            out[gi] = fma_t<T>(-alpha_s, vec_of<T>(x, s_cur), w1);
-            a.psi[gi] = fma_t<T>(y_s, x, a.psi[gi]);
-          }
+          const T w1 = mul_t<T>(acc[i][u], s_cur);
+          out[gi] = w1;
+          dot = fma_t<T>(vec_of<T>(g[gi], s_cur), w1, dot);
         }
       }
     }
@@ -1512,8 +1494,6 @@ static ed_status prepare_passa() {
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
   ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_LANCZOS, true, true, RT, NT>,
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
-  ED_TRY_CUDA(cudaFuncSetAttribute(k_hv<T, HV_SECOND, true, true, RT, NT>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HV_SMEM_MAX));
   return ED_OK;
 }
 
@@ -1553,10 +1533,13 @@ template ed_status ed_hv_prepare<double>();
 template <typename T, int MODE>
 static void launch_dw(const HvLaunch<T> &a, unsigned ns, cudaStream_t st) {
   const dim3 grid((unsigned)a.tb.nditems, ns);
-  if (a.tb.dw_narrow)
-    k_hv_dw<T, MODE, 1, 4><<<grid, DW_THREADS, 0, st>>>(a);
-  else
-    k_hv_dw<T, MODE, Tile<T>::RT, 2><<<grid, DW_THREADS, 0, st>>>(a);
+  if constexpr (sizeof(T) == 4) {
+    if (a.tb.dw_narrow) {
+      k_hv_dw<T, MODE, 1, 4><<<grid, DW_THREADS, 0, st>>>(a);
+      return;
+    }
+  }
+  k_hv_dw<T, MODE, Tile<T>::RT, 2><<<grid, DW_THREADS, 0, st>>>(a);
 }
 
 template <typename T, int MODE>
@@ -1575,20 +1558,24 @@ static ed_status launch_mode(const HvLaunch<T> &a, unsigned ns, cudaStream_t st)
       k_hv_small<T, MODE, true><<<grid, HVS_THREADS, 0, st>>>(a);
     else
       k_hv_small<T, MODE, false><<<grid, HVS_THREADS, 0, st>>>(a);
-  } else if (a.tb.fiber) {
-    if constexpr (sizeof(T) == 4) {
-      ED_TRY(launch_fiber(a.tb.fiber, &a, ed_hv_plain(MODE) ? HV_PLAIN : MODE, ns, st));
-    }
-    launch_dw<T, MODE>(a, ns, st);
   } else if (a.tb.ditems) {
-    if (a.tb.passa_wide)
-      k_hv<T, MODE, true, true, rt_passa<T, true>(), passa_threads<true>()>
-          <<<dim3((unsigned)a.tb.nitems, ns), passa_threads<true>(), a.tb.smem, st>>>(a);
-    else
-      k_hv<T, MODE, true, true, rt_passa<T, false>(), passa_threads<false>()>
-          <<<dim3((unsigned)a.tb.nitems, ns), passa_threads<false>(), a.tb.smem, st>>>(a);
-    ED_LAUNCHED(1);
-    launch_dw<T, MODE>(a, ns, st);
+    if constexpr (MODE == HV_SECOND) {
+      return ED_ERR_ARG;  // see second_pass
+    } else {
+      if (a.tb.fiber) {
+        if constexpr (sizeof(T) == 4)
+          ED_TRY(launch_fiber(a.tb.fiber, &a, ed_hv_plain(MODE) ? HV_PLAIN : MODE, ns, st));
+      } else {
+        if (a.tb.passa_wide)
+          k_hv<T, MODE, true, true, rt_passa<T, true>(), passa_threads<true>()>
+              <<<dim3((unsigned)a.tb.nitems, ns), passa_threads<true>(), a.tb.smem, st>>>(a);
+        else
+          k_hv<T, MODE, true, true, rt_passa<T, false>(), passa_threads<false>()>
+              <<<dim3((unsigned)a.tb.nitems, ns), passa_threads<false>(), a.tb.smem, st>>>(a);
+        ED_LAUNCHED(1);
+      }
+      launch_dw<T, MODE>(a, ns, st);
+    }
   } else if (a.tb.ell_col) {
     k_hv<T, MODE, true><<<dim3((unsigned)a.tb.nitems, ns), HV_THREADS, a.tb.smem, st>>>(a);
   } else {
