@@ -201,8 +201,8 @@ ed_status ed_sector_blocked_kernel(ed_sector s, ed_precision prec, int32_t *kern
 
 /* Autotuner (no counterpart in the paper).  Sectors of at most 2^17 padded
  * elements use the element-parallel kernel; above that the first sector of
- * each model shape (Norb, Nbath, precision) and, in FP32, of each factor of 8
- * in padded elements (2^17, 2^20, 2^23, ..) times the tiled family and
+ * each model shape (Norb, Nbath, precision) and, in FP32, of each size (below
+ * 2^20 padded elements, below 13 * 2^20, above) times the tiled family and
  * the element-parallel kernel (one warm-up and three launches each, on two
  * scratch vectors of the sector's size) when its block-major tables are
  * built, and every sector of that shape and size in the process then uses the
@@ -213,8 +213,9 @@ ed_status ed_sector_blocked_kernel(ed_sector s, ed_precision prec, int32_t *kern
  * kernel for one sector and precision: ED_KERNEL_ELEMENTWISE or the tiled
  * family (ED_KERNEL_TILED, or
  * ED_KERNEL_TWO_PASS where the block sizes call for two passes); other
- * requests give ED_ERR_UNSUPPORTED.  ed_matvec follows a pin as described there.  All kernels compute the same w = H v bit
- * for bit; Lanczos runs differ only in the summation order of <v, w>. */
+ * requests give ED_ERR_UNSUPPORTED.  ed_matvec follows a pin as described
+ * there.  All kernels compute the same w = H v bit for bit; Lanczos runs differ
+ * only in the summation order of <v, w>. */
 ed_status ed_sector_tune_info(ed_sector s, ed_precision prec, int32_t *kernel, double *host_ms);
 ed_status ed_sector_set_kernel(ed_sector s, ed_precision prec, int32_t kernel);
 ed_status ed_sector_permute(ed_sector s, ed_precision prec, int32_t to_blocked,
@@ -225,7 +226,11 @@ typedef struct {
   ed_precision precision;
   int32_t max_iter;      /* first-pass Lanczos steps, <= ED_MAX_LANCZOS (0: 512) */
   double tol;            /* stop when beta_{k+1}|y_k| <= tol*max(1,|theta|)      */
-                         /* (0: 1e-12 for FP64, 1e-6 for the FP32 modes)         */
+                         /* (0: 1e-12 for FP64, 1e-6 for the FP32 modes); tested */
+                         /* on some steps only, and on earlier ones where rounding
+                            has brought a copy of the converged state since: then
+                            `iterations` is the earlier step, `matvecs` counts the
+                            products run                                          */
   uint64_t seed;         /* start vector: v0_i = u_i - 1/2, u_i = SplitMix64(seed)
                             output i, sector order, then normalised               */
   int32_t polish_steps;  /* FP64 Lanczos steps of ED_FP32_POLISH (0: 4)          */

@@ -53,16 +53,14 @@ constexpr bool ed_takes_permuted(int norb, int group, int64_t dim, int64_t bdim,
 // Size class of the autotuner's key.  Sectors of at most 2^17 padded elements
 // are not timed.  In FP32 the faster kernel of a model shape changes with the
 // size (element-parallel / tiled ms: Norb=2 Ns=14 0.5 at 1e6 elements, 1.3 at
-// 1.2e7; Norb=3 0.25 at Ns=12, 2.3 at Ns=18), so a class spans a factor of 8:
-// over the 509 sectors of 15 shapes within three electrons of half filling,
-// the choice of a class's first sector costs the others 1.9% on average (3.6%
-// with one class per shape, and up to 3.1 times).  In FP64 the
-// element-parallel kernel was the faster one throughout: one class, no further
-// timing.
+// 1.2e7; Norb=3 0.25 at Ns=12, 2.3 at Ns=18), so there are three classes: over
+// 457 sectors of 15 shapes within three electrons of half filling, the choice
+// of a class's first sector costs the others 2.2% on average (3.6% with one
+// class per shape, up to 3.1 times; 1.9% with a class per factor of 8, whose
+// boundaries run between the half-filled sector of an odd Ns and its
+// neighbours: a solve would time both).  In FP64 the element-parallel kernel was
+// the faster one throughout: one class, no further timing.
 constexpr int64_t ED_TUNE_MIN = (int64_t)1 << 17;
 constexpr int ed_tune_class(int elem, int64_t bdim) {
-  int c = 0;
-  if (elem == 4)
-    for (bdim /= ED_TUNE_MIN * 8; bdim > 0; bdim /= 8) ++c;
-  return c;
+  return elem != 4 ? 0 : (bdim >= (int64_t)1 << 20) + (bdim >= (int64_t)13 << 20);
 }

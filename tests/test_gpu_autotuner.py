@@ -1,4 +1,4 @@
-"""The autotuner's choice holds for a model shape within a factor of 8 in size."""
+"""The autotuner's choice holds for a model shape and a class of sizes."""
 import pytest
 
 from workloads import make_model
