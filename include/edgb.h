@@ -144,8 +144,9 @@ ed_status ed_sector_free(ed_sector s);
  * Asynchronous on `stream`.
  *
  * Large FP32 sectors of several orbitals go through block-major order where
- * that is the faster way (from 2^25 elements with two or three orbitals, 2^27
- * with four; from 2^20 where ed_sector_set_kernel pinned the tiled family),
+ * that is the faster way (from 2^20 elements on: two to four orbitals with
+ * long rows, D_up of some thousand or more; or wherever ed_sector_set_kernel
+ * pinned the tiled family),
  * in a scratch of two vectors, at most 2 GiB, that returns to the library's
  * pool (ed_memory_trim).  Without memory for it, and on a stream under
  * capture, the sector-order kernel serves the call: the same sum of the same

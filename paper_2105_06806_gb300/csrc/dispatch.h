@@ -27,13 +27,17 @@ constexpr bool ed_takes_rows(int elem, int64_t ddw, int64_t stride) {
 
 // Sector-order FP32 product through block-major order (two permutations and
 // the orbital-factorised product in a scratch pair of vectors) instead of the
-// sector-order kernel, whose H_up hops gather across whole CSR rows.  Measured
-// on every sector within two electrons of half filling, sector-order kernel /
-// detour in us: two orbitals at Ns=16 1019 / 751 to 2724 / 1950 (9 sectors of
-// 9 faster), three at Ns=15 from 2^25 elements 714 / 570; below 2^25 elements
-// between 0.85 and 1.15 times, and mostly slower (Norb=2 Ns=14 (7,7) 146 / 158,
-// Norb=3 Ns=15 (5,7) 257 / 269); four orbitals 2542 / 2420 from 2^27
-// elements, below that 0.95 to 1.1 times; five orbitals 704 / 840.
+// sector-order kernel, whose H_up hops gather across whole CSR rows and cost
+// the more the longer those are (D_up).  Sector-order kernel / detour, measured
+// on 230 sectors of Ns=14-20, with and without exchange terms:
+//   two, three orbitals: D_up from 8008 on 1.06 to 1.9 (Norb=2 Ns=16 (8,8) 2724
+//     / 1950 us; 2.1 to 4.0 with two down electrons), with fewer than 5 * 2^20
+//     elements only from 11440 on (8008: 0.93); 5005 and 6435 from 5 * 2^20
+//     elements on 1.0 to 1.43, below that down to 0.83; up to 3432 0.85 to 1.24
+//     either way (Norb=2 Ns=14 (7,7) 146 / 158 us, Norb=3 Ns=15 (5,7) 257 / 269);
+//   four orbitals: D_up from 12870 on 1.01 to 3.6, 11440 from 2^25 elements on
+//     1.01 to 1.1, below that and with shorter rows 0.70 to 0.99;
+//   five orbitals: 0.59 to 0.84 without exchange terms, 0.86 to 1.2 with them.
 // group: levels of an orbital group, 0 where the factorised product does not
 // apply; pinned: the kernel the caller chose for the block-major layout (0 the
 // tiled family, which is then taken from 2^20 elements on, 1 element-parallel,
@@ -42,12 +46,14 @@ constexpr bool ed_takes_rows(int elem, int64_t ddw, int64_t stride) {
 constexpr int64_t ED_PERMUTE_MIN = (int64_t)1 << 20;
 constexpr int64_t ED_PERMUTE_SCRATCH_MAX = (int64_t)2 << 30;
 constexpr int64_t ed_permute_scratch(int64_t bdim) { return 2 * bdim * (int64_t)sizeof(float); }
-constexpr bool ed_takes_permuted(int norb, int group, int64_t dim, int64_t bdim, int pinned) {
+constexpr bool ed_takes_permuted(int norb, int group, int64_t dup, int64_t dim, int64_t bdim,
+                                 int pinned) {
   if (group == 0 || dim < ED_PERMUTE_MIN || pinned == 1 ||
       ed_permute_scratch(bdim) > ED_PERMUTE_SCRATCH_MAX)
     return false;
   if (pinned == 0) return true;
-  return norb <= 3 ? dim >= (int64_t)1 << 25 : norb == 4 && dim >= (int64_t)1 << 27;
+  if (norb <= 3) return dup >= (dim >= (int64_t)5 << 20 ? 5000 : 11000);
+  return norb == 4 && dup >= (dim >= (int64_t)1 << 25 ? 11000 : 12000);
 }
 
 // Size class of the autotuner's key.  Sectors of at most 2^17 padded elements

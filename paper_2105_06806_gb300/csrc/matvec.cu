@@ -1649,7 +1649,8 @@ static ed_status matvec_permuted(ed_sector s, const float *v, float *w, cudaStre
   *done = false;
   if (s->mp.norb < 2 || s->dim < ED_PERMUTE_MIN) return ED_OK;
   const int pinned = s->hv_pinned[0] ? s->hv_kernel[0] : -1;
-  if (!ed_takes_permuted(s->mp.norb, fiber_group(s), s->dim, s->bdim, pinned) || capturing(st))
+  if (!ed_takes_permuted(s->mp.norb, fiber_group(s), s->sp[0].dim, s->dim, s->bdim, pinned) ||
+      capturing(st))
     return ED_OK;
   // the sector-order list too, so that a later call under capture builds nothing
   ED_TRY(ed_build_items(s, 0, 4));

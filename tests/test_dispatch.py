@@ -48,26 +48,32 @@ def test_rows_kernel_within_its_32_bit_units(tmp_path):
 def test_sector_order_detour_rule(tmp_path):
     """The sector-order FP32 product goes through block-major order only where that was
     measured faster, never with a scratch above 2 GiB, and follows a pinned kernel."""
-    G = 1 << 30
-    cases = [  # norb, group, dim, bdim, pinned, want
-        (2, 7, 11778624, 11806080, -1, 0),      # Norb=2 Ns=14 (7,7): slower
-        (2, 8, 165636900, 165791340, -1, 1),    # Norb=2 Ns=16 (8,8)
-        (3, 5, 41409225, 41460705, -1, 1),      # Norb=3 Ns=15 (7,7)
-        (3, 5, 15030015, 15100000, -1, 0),
-        (4, 4, 165636900, 166000000, -1, 1), (4, 4, 102951200, 103200000, -1, 0),
-        (5, 3, 41409225, 41900000, -1, 0),      # five orbitals: never faster
-        (2, 0, 2363904400, 2364000000, -1, 0),  # groups the factorised product does not take
-        (3, 6, 2363904400, 2364487840, -1, 0),  # Norb=3 Ns=18: 19 GB of scratch
-        (3, 6, 2363904400, 2364487840, 0, 0),
-        (2, 8, G // 4, G // 4, -1, 1), (2, 8, G // 4, G // 4 + 1, -1, 0),
-        (2, 8, 1 << 25, 1 << 25, -1, 1), (2, 8, (1 << 25) - 1, 1 << 25, -1, 0),
-        (4, 4, 1 << 27, 1 << 27, -1, 1), (4, 4, (1 << 27) - 1, 1 << 27, -1, 0),
-        (2, 7, 6012006, 6030000, 0, 1), (2, 7, (1 << 20) - 1, 1 << 20, 0, 0),  # tiled pinned
-        (5, 3, 1 << 20, 1 << 20, 0, 1), (2, 8, 165636900, 165791340, 1, 0),    # pinned
+    M, G = 1 << 20, 1 << 30
+    cases = [  # norb, group, dup, dim, bdim, pinned, want
+        (2, 7, 3432, 11778624, 11806080, -1, 0),   # Norb=2 Ns=14 (7,7): slower
+        (2, 8, 12870, 165636900, 165791340, -1, 1),  # Norb=2 Ns=16 (8,8)
+        (3, 5, 6435, 41409225, 41460705, -1, 1),   # Norb=3 Ns=15 (7,7)
+        (3, 5, 5005, 15030015, 15100000, -1, 1),
+        (3, 5, 3003, 19324305, 19400000, -1, 0),
+        (4, 4, 11440, 91611520, 92000000, -1, 1), (4, 4, 8008, 102951200, 103200000, -1, 0),
+        (4, 4, 12870, 7207200, 7300000, -1, 1),
+        (5, 3, 6435, 41409225, 41900000, -1, 0),   # five orbitals
+        (2, 0, 48620, 200000000, 201000000, -1, 0),  # no factorised product
+        (3, 6, 48620, 2363904400, 2364487840, -1, 0),  # Norb=3 Ns=18: 19 GB of scratch
+        (3, 6, 48620, 2363904400, 2364487840, 0, 0),
+        (2, 8, 8008, G // 4, G // 4, -1, 1), (2, 8, 8008, G // 4, G // 4 + 1, -1, 0),
+        (2, 8, 5000, 5 * M, 5 * M, -1, 1), (2, 8, 5000, 5 * M - 1, 5 * M, -1, 0),
+        (2, 8, 4999, 5 * M, 5 * M, -1, 0), (2, 8, 11000, M, M, -1, 1),
+        (2, 8, 11000, M - 1, M, -1, 0),
+        (4, 4, 11000, 32 * M, 32 * M, -1, 1), (4, 4, 11000, 32 * M - 1, 32 * M, -1, 0),
+        (4, 4, 12000, 32 * M - 1, 32 * M, -1, 1), (4, 4, 10999, 32 * M, 32 * M, -1, 0),
+        (2, 7, 2002, 6012006, 6030000, 0, 1), (2, 7, 2002, M - 1, M, 0, 0),  # tiled pinned
+        (5, 3, 3003, M, M, 0, 1), (2, 8, 12870, 165636900, 165791340, 1, 0),  # pinned
     ]
-    got = _run(tmp_path, "\n".join('printf("%%d\\n", (int)ed_takes_permuted(%d, %d, %dLL, %dLL, %d));'
-                                   % c[:5] for c in cases))
-    assert got == [c[5] for c in cases]
+    got = _run(tmp_path, "\n".join(
+        'printf("%%d\\n", (int)ed_takes_permuted(%d, %d, %dLL, %dLL, %dLL, %d));' % c[:6]
+        for c in cases))
+    assert got == [c[6] for c in cases]
 
 
 def test_size_classes_of_the_autotuner(tmp_path):
