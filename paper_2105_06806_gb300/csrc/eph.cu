@@ -244,7 +244,7 @@ extern "C" ed_status ed_eph_matvec(ed_sector s, const ed_phonon *ph, ed_precisio
   }
   cudaStream_t cs = (cudaStream_t)stream;
   int layout = 0;
-  ED_TRY(ed_sector_order_layout(s, prec == ED_FP64 ? 8 : 4, d_v, d_w, cs, &layout));
+  ED_TRY(ed_sector_order_layout(s, prec, d_v, d_w, cs, &layout));
   if (prec == ED_FP64) {
     ED_TRY(ed_build_items(s, layout, 8));
     return eph_apply<double>(s, pp, layout, (const double *)d_v, (double *)d_w, cs);

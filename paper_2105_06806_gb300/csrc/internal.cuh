@@ -461,7 +461,8 @@ inline bool ed_same_layout(ed_sector s) { return s->mp.norb == 1 && s->bstride =
 // for bit), whose tables the first such call builds.  Where that fails (no
 // memory for the tables or the autotuner's vectors) or the stream is under
 // capture, 0: the sector-order kernel needs its own list alone.
-ed_status ed_sector_order_layout(ed_sector s, int elem, const void *v, const void *w,
+// ED_ERR_ARG for an unknown precision, before anything is built.
+ed_status ed_sector_order_layout(ed_sector s, ed_precision prec, const void *v, const void *w,
                                  cudaStream_t st, int *layout);
 
 int64_t ed_hv_num_parts(ed_sector s, int layout, int elem_size);

@@ -1676,9 +1676,11 @@ static ed_status matvec_permuted(ed_sector s, const float *v, float *w, cudaStre
   return rs;
 }
 
-ed_status ed_sector_order_layout(ed_sector s, int elem, const void *v, const void *w,
+ed_status ed_sector_order_layout(ed_sector s, ed_precision prec, const void *v, const void *w,
                                  cudaStream_t st, int *layout) {
   *layout = 0;
+  if (prec != ED_FP64 && prec != ED_FP32 && prec != ED_FP32_POLISH) return ED_ERR_ARG;
+  const int elem = prec == ED_FP64 ? 8 : 4;
   if (!ed_same_layout(s) || (((uintptr_t)v | (uintptr_t)w) & 15)) return ED_OK;
   // the sector-order list too, so that a later call under capture builds nothing
   ED_TRY(ed_build_items(s, 0, elem));
@@ -1710,7 +1712,7 @@ static ed_status matvec_layout(ed_sector s, ed_precision prec, const void *d_v, 
     return ED_ERR_ARG;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  if (layout == 0) ED_TRY(ed_sector_order_layout(s, prec == ED_FP64 ? 8 : 4, d_v, d_w, st, &layout));
+  if (layout == 0) ED_TRY(ed_sector_order_layout(s, prec, d_v, d_w, st, &layout));
   if (prec == ED_FP64) {
     ED_TRY(ed_build_items(s, layout, 8));
     return ed_launch_hv<double>(s, ed_hv_tables<double>(s, layout), HV_PLAIN,

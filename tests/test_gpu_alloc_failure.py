@@ -163,3 +163,17 @@ def test_one_orbital_product_under_capture(ed):
     torch.cuda.synchronize()
     assert torch.equal(w, y)
     s.free()
+
+
+def test_unknown_precision_builds_nothing(ed):
+    """Refused before the first allocation, as an argument error."""
+    s = ed.Sector(make_model(1, 11, U=2.0, seed=4), 6, 5)
+    v, w = _vec(s.dim, torch.float64), torch.empty(s.dim, device="cuda", dtype=torch.float64)
+    ed.inject_alloc_failure(1)
+    for product in (lambda: ed.matvec(s, v, w, 7),
+                    lambda: ed.eph_matvec(s, ed.phonon(0.5, [0.3], 0), v, w, 7)):
+        with pytest.raises(ed.EDError) as e:
+            product()
+        assert e.value.status == ed.ED_ERR_ARG
+    ed.inject_alloc_failure(0)
+    s.free()
